@@ -76,8 +76,9 @@ typedef struct {
   int flow;            /* KD_FLOW_*; NONE (u = 0) leaves pure diffusion */
   int n;               /* fine grid side, even (kept set |kx|, |ky| <= n/3).  KD_FINE_FFT:
                           n = 16, 32, ..., 1024 and 96, 160, 192 (32 R, R = 3, 5, 6: mixed
-                          radix; Table 1's N_F = 160) transform on n itself; any other even
-                          n <= 286 on the smallest mixed-radix side m >= 2 (n/3) + 2: the flow
+                          radix; Table 1's N_F = 160) transform on n itself (the default
+                          complex64 plans of n = 512 and 1024 on 3n/4 points, by the rule
+                          that follows); any other even n <= 286 on the smallest mixed-radix side m >= 2 (n/3) + 2: the flow
                           has only the wavenumbers +-1, so m points resolve u x b on the kept
                           set without aliasing, exactly as n points do (n = 240, the 3/2-padded
                           grid of 160 kept modes, runs on m = 192).  KD_FINE_CONV: even

@@ -24,10 +24,13 @@
 //                     9 = 512-point warp transforms, one warp per component of a row
 //                     (kd_fine5.cuh; n = 512)
 //   n = 1024  column: 4 = warp-owned transforms (kd_fine4.cuh), one warp per component,
-//                     4 columns per block; 5 = warp-owned transforms, one warp per column,
-//                     8 columns per block; 6 = the same with two independent groups of
-//                     4 columns per block
+//                     4 columns per block; 5, 6 = warp-owned transforms, one warp per column,
+//                     8 columns per block
 //             row:    7 = warp-owned transforms, one row per block
+//   The default pairs (column 6, row 7) at n = 1024 and (5, 9) at n = 512 step RK443 on 3n/4
+//   points with the kernels of kd_narrow.cuh (the two kernels of a plan share the mixed
+//   field's grid, so they come as a pair); with another partner or scheme, these indices are
+//   the n-point kernels above.
 #pragma once
 #include "kd_fine2c.cuh"
 #include "kd_fine3.cuh"
@@ -35,6 +38,7 @@
 #include "kd_fine2f.cuh"
 #include "kd_fine4.cuh"
 #include "kd_fine5.cuh"
+#include "kd_narrow.cuh"
 #include "kd_fine_mr.cuh"
 
 namespace kd {
@@ -64,6 +68,7 @@ struct FineMrSet {
   static constexpr int N = 32 * R;
   static constexpr bool FUSED = false;
   static constexpr int kFusedCol = -1;
+  static constexpr bool narrow(int, int, int) { return false; }
   static constexpr unsigned BLOCK = 32 * kMrWarps;
   static int ncol() { return 1; }
   static int nrow() { return 1; }
@@ -228,6 +233,7 @@ struct Fine2Set {
   // variant does not apply)
   static constexpr bool FUSED = WIDE && N == 128;
   static constexpr int kFusedCol = 4;
+  static constexpr bool narrow(int, int, int) { return false; }
   // the warp-owned mixed-radix kernels (FineMrSet) as a further column / row variant of
   // the sides 32 R, complex64 (complex128 keeps one plan: the serial fine run, tuned for
   // one field, and the batched sweeps then take the same kernels, so a Parareal run of N
@@ -369,6 +375,55 @@ static cudaError_t prepare_row4() {
                               (int)G::smem);
 }
 
+// Kernels on N = 3n/4 points (kd_narrow.cuh): column kernel with kNarrowGroups groups a
+// block, one block per SM; row kernel with as many blocks per SM as fit.
+constexpr int kNarrowVariant = 100, kNarrowGroups = 3;
+
+template <int N>
+static void launch_coln(const FineArgs& a, int s, int j, cudaStream_t st, bool pdl) {
+  using C = ColN<N, kNarrowGroups>;
+  const long groups = (long)a.batch * (N / C::XG);
+  launch_k(coln_kernel<N, kNarrowGroups>, persistent_grid((groups + C::GR - 1) / C::GR), C::BLOCK, C::smem, st, pdl, a,
+           s, j);
+}
+
+template <int N, int MODE>
+static void launch_rown_mode(const FineArgs& a, int store, cudaStream_t st, bool pdl) {
+  using G = RowN<N, MODE>;
+  const long blocks = ((long)a.batch * a.P + G::W::C - 1) / G::W::C;
+  const long cap = (long)persistent_grid(1L << 30) * G::MINB;
+  launch_k(rown_kernel<N, MODE>, (unsigned)(blocks < cap ? blocks : cap), G::BLOCK, G::smem, st, pdl, a, store);
+}
+
+template <int N>
+static void launch_rown(const FineArgs& a, int mode, int store, cudaStream_t st, bool pdl) {
+  switch (mode) {
+    case 0: return launch_rown_mode<N, 0>(a, store, st, pdl);
+    case 1: return launch_rown_mode<N, 1>(a, store, st, pdl);
+    case 2: return launch_rown_mode<N, 2>(a, store, st, pdl);
+    case 3: return launch_rown_mode<N, 3>(a, store, st, pdl);
+    default: return launch_rown_mode<N, 4>(a, store, st, pdl);
+  }
+}
+
+template <int N, int MODE>
+static cudaError_t prepare_rown() {
+  return cudaFuncSetAttribute(rown_kernel<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)RowN<N, MODE>::smem);
+}
+
+template <int N>
+static cudaError_t prepare_narrow() {
+  cudaError_t e = cudaFuncSetAttribute(coln_kernel<N, kNarrowGroups>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)ColN<N, kNarrowGroups>::smem);
+  if (e == cudaSuccess) e = prepare_rown<N, 0>();
+  if (e == cudaSuccess) e = prepare_rown<N, 1>();
+  if (e == cudaSuccess) e = prepare_rown<N, 2>();
+  if (e == cudaSuccess) e = prepare_rown<N, 3>();
+  if (e == cudaSuccess) e = prepare_rown<N, 4>();
+  return e;
+}
+
 template <typename T, int N>
 struct Fine3Set {
   using Sh = Shapes3<T, N>;
@@ -381,6 +436,11 @@ struct Fine3Set {
   static constexpr int XTC = Sh::XT0, RTC0 = Sh::RT0, RTC1 = Sh::RT0 / 2;
   static constexpr bool FUSED = false;   // no persistent fused step at these sizes
   static constexpr int kFusedCol = -1;
+  // the pair of variants that steps on NN = 3n/4 points
+  static constexpr int NN = N / 4 * 3;
+  static constexpr bool narrow(int col, int row, int scheme) {
+    return scheme == SCHEME_RK443 && ((W4 && col == kW6Col && row == kW4Row) || (R8 && col == kC512Col && row == kC512Row));
+  }
   static int ncol() { return WIDE ? (R8 ? 6 : (W4 ? 7 : 4)) : 1; }
   // plan of a context that is not autotuned: the warp-transform kernels where they exist
   static FinePlan default_plan() {
@@ -400,15 +460,15 @@ struct Fine3Set {
     if constexpr (R8) {
       if ((e = prepare_w<N>()) != cudaSuccess) return e;
     }
+    if constexpr (R8 || W4) {
+      if ((e = prepare_narrow<NN>()) != cudaSuccess) return e;
+    }
     if constexpr (W4) {
       if ((e = cudaFuncSetAttribute(col4_kernel<N, kCol4Copy>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)Col4<N, kCol4Copy>::smem)) != cudaSuccess)
         return e;
       if ((e = cudaFuncSetAttribute(col5_kernel<N, 8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)Col5<N, 8, 1>::smem)) != cudaSuccess)
-        return e;
-      if ((e = cudaFuncSetAttribute(col5_kernel<N, 4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)Col5<N, 4, 2>::smem)) != cudaSuccess)
         return e;
       if ((e = prepare_row4<N, 0>()) != cudaSuccess) return e;
       if ((e = prepare_row4<N, 1>()) != cudaSuccess) return e;
@@ -451,17 +511,14 @@ struct Fine3Set {
     return cudaSuccess;
   }
   static void col(int v, const FineArgs& a, int s, int j, cudaStream_t st, bool pdl) {
+    if constexpr (R8 || W4) {
+      if (v == kNarrowVariant) return launch_coln<NN>(a, s, j, st, pdl);
+    }
     if constexpr (W4) {
-      if (v == kW5Col) {
+      if (v == kW5Col || v == kW6Col) {
         using C5 = Col5<N, 8, 1>;
         launch_k(col5_kernel<N, 8, 1>, persistent_grid((long)a.batch * (N / C5::XG)), C5::BLOCK, C5::smem, st, pdl,
                  a, s, j);
-        return;
-      }
-      if (v == kW6Col) {
-        using C6 = Col5<N, 4, 2>;
-        const long groups = (long)a.batch * (N / C6::XG);
-        launch_k(col5_kernel<N, 4, 2>, persistent_grid((groups + 1) / 2), C6::BLOCK, C6::smem, st, pdl, a, s, j);
         return;
       }
       if (v == kW4Col) {
@@ -489,6 +546,9 @@ struct Fine3Set {
     }
   }
   static void row(int v, const FineArgs& a, int mode, int store, cudaStream_t st, bool pdl) {
+    if constexpr (R8 || W4) {
+      if (v == kNarrowVariant) return launch_rown<NN>(a, mode, store, st, pdl);
+    }
     if (!WIDE) v = 0;
     if (a.scheme == SCHEME_RK222) return launch_row3<T, N, Sh::rt(0), true, 16, SCHEME_RK222>(a, mode, store, st, pdl);
     if (a.scheme == SCHEME_RK111) return launch_row3<T, N, Sh::rt(0), true, 16, SCHEME_RK111>(a, mode, store, st, pdl);
@@ -536,7 +596,8 @@ static int run_steps(const FineArgs& a0, const StepCfg& cfg) {
   if constexpr (Set::FUSED) {
     if (cv == Set::kFusedCol) cv = 0;   // (only for the calls the fused step does not cover)
   }
-  const int rv = pl.row >= 0 && pl.row < Set::nrow() ? pl.row : 0;
+  int rv = pl.row >= 0 && pl.row < Set::nrow() ? pl.row : 0;
+  if (Set::narrow(cv, rv, a0.scheme)) cv = rv = kNarrowVariant;
   int launches = 0;
   if constexpr (Set::FUSED) {
     // the persistent fused step: every step of every field in one launch (RK443, from X,

@@ -75,13 +75,15 @@ enum { KD_RK443 = 0, KD_RK222 = 1, KD_RK111 = 2 };
 typedef struct {
   int flow;            /* KD_FLOW_*; NONE (u = 0) leaves pure diffusion */
   int n;               /* fine grid side, even (kept set |kx|, |ky| <= n/3).  KD_FINE_FFT:
-                          n = 16, 32, ..., 1024 and 96, 160, 192 (32 R, R = 3, 5, 6: mixed
-                          radix; Table 1's N_F = 160) transform on n itself (the default
-                          complex64 plans of n = 512 and 1024 on 3n/4 points, by the rule
-                          that follows); any other even n <= 286 on the smallest mixed-radix side m >= 2 (n/3) + 2: the flow
-                          has only the wavenumbers +-1, so m points resolve u x b on the kept
-                          set without aliasing, exactly as n points do (n = 240, the 3/2-padded
-                          grid of 160 kept modes, runs on m = 192).  KD_FINE_CONV: even
+                          n = 16, 32, ..., 1024 or any other even n <= 286.  The flow has only
+                          the wavenumbers +-1, so any m >= 2 (n/3) + 2 points resolve u x b on
+                          the kept set without aliasing, exactly as n points do, and RK443
+                          steps transform on such an m: 24, 32, 48, 96, 128 or 192 for n <= 286,
+                          3n/4 for n = 512 and 1024 in complex64 (n = 240, the 3/2-padded grid
+                          of 160 kept modes, runs on 192); complex128 n = 256, 512 and 1024,
+                          launch plans other than the default, RK222 and RK111 on n
+                          itself or, where n is neither a power of two nor 96, 160, 192, on the
+                          smallest of these three that suffices.  KD_FINE_CONV: even
                           n <= 190 */
   double kz;           /* wavenumber along the invariant direction (the paper's kx for GP) */
   double Rm;           /* magnetic Reynolds number (Eq. 2), > 0 */

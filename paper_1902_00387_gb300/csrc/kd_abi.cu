@@ -254,17 +254,24 @@ kd_status with_phases(kd_ctx* ctx, FineWs& w, FineArgs& a, int nsteps) {
 }
 
 int run_fine(kd_ctx* ctx, int g, int prec, const FineArgs& a, int nsteps, bool prologue, bool store_last,
-             const LaunchProbe* probe, const int* active) {
+             const LaunchProbe* probe, const int* active, const FinePlan* plan) {
   StepCfg cfg;
   cfg.nsteps = nsteps;
   cfg.prologue = prologue;
   cfg.store_last = store_last;
   cfg.active = active;
   cfg.probe = probe;
-  cfg.plan = ctx->plan[g];
+  cfg.plan = plan ? *plan : ctx->plan[g];
   cfg.pdl = ctx->pdl != 0;
   cfg.st = ctx->st;
   return fine_run(prec, a, cfg);
+}
+
+FinePlan call_plan(const kd_ctx* ctx, long batch) {
+  const int n = ctx->p.n, prec = ctx->p.prec_fine;
+  const FinePlan d = fine_default_plan(n, prec);
+  const bool is_default = ctx->plan[0].col == d.col && ctx->plan[0].row == d.row;
+  return is_default && batch <= fine_few(n, prec) ? fine_default_plan(n, prec, true) : ctx->plan[0];
 }
 
 kd_status ensure_full_tmp(kd_ctx* ctx, size_t bytes) {
@@ -765,7 +772,7 @@ kd_status kd_create(const kd_params* params, void* cuda_stream, kd_ctx** out) {
   kd_ctx* ctx = new kd_ctx();
   ctx->p = *params;
   ctx->plan[0] = fine_default_plan(params->n, params->prec_fine);
-  ctx->plan[1] = fine_default_plan(params->n_coarse, params->prec_coarse);
+  ctx->plan[1] = fine_default_plan(params->n_coarse, params->prec_coarse, true);
   if (params->learned_modes > 0) {
     ctx->cK = params->learned_modes / 2;
     ctx->cP = params->learned_modes;
@@ -775,8 +782,8 @@ kd_status kd_create(const kd_params* params, void* cuda_stream, kd_ctx** out) {
   }
   ctx->st = (cudaStream_t)cuda_stream;
   cudaError_t e = cudaGetDevice(&ctx->device);
-  if (e == cudaSuccess) e = fine_prepare(params->prec_fine);
-  if (e == cudaSuccess) e = fine_prepare(params->prec_coarse);
+  if (e == cudaSuccess) e = fine_prepare(params->prec_fine, params->n);
+  if (e == cudaSuccess) e = fine_prepare(params->prec_coarse, params->n_coarse);
   if (e == cudaSuccess) e = coarse_prepare(params->prec_coarse);
   if (e == cudaSuccess && params->fine_operator == KD_FINE_CONV) e = coarse_prepare(params->prec_fine);
   for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreate(&ctx->ev[i]);
@@ -861,8 +868,17 @@ kd_status kd_destroy(kd_ctx* ctx) {
   return KD_OK;
 }
 
+static kd_status fine_full(kd_ctx* ctx, const void* b_in, void* b_out, const double* t0, int nsteps, int batch,
+                           const FinePlan& plan);
+static kd_status fine_kept(kd_ctx* ctx, const void* c_in, void* c_out, const double* t0, int nsteps, int batch,
+                           const FinePlan& plan);
+
 kd_status kd_fine_batched(kd_ctx* ctx, const void* b_in, void* b_out, const double* t0, int nsteps, int batch) {
-  if (!ctx) return KD_EINVAL;
+  return ctx ? fine_full(ctx, b_in, b_out, t0, nsteps, batch, call_plan(ctx, batch)) : KD_EINVAL;
+}
+
+static kd_status fine_full(kd_ctx* ctx, const void* b_in, void* b_out, const double* t0, int nsteps, int batch,
+                           const FinePlan& plan) {
   if (!b_in || !b_out || !t0) return fail(ctx, KD_EINVAL, "kd_fine_batched: NULL buffer");
   if (batch < 0 || nsteps < 0) return fail(ctx, KD_EINVAL, "kd_fine_batched: negative batch or nsteps");
   if (batch == 0) return KD_OK;
@@ -880,7 +896,7 @@ kd_status kd_fine_batched(kd_ctx* ctx, const void* b_in, void* b_out, const doub
   // kernels that take the state in the caller's layout skip the pack and unpack passes:
   // the first step reads b_in, the last writes the kept entries of b_out, and the rest of
   // b_out is zeroed (b_in == b_out is fine: a row is read before it is written)
-  const bool full_io = nsteps > 0 && fine_full_io(n, pf, ctx->plan[0], ctx->p.fine_scheme);
+  const bool full_io = nsteps > 0 && fine_full_io(n, pf, plan, ctx->p.fine_scheme);
   if (!full_io) KD_LAUNCH(full_to_compact(pf, b_in, pf, ctx->ws_f.X, batch, n, ctx->st), "pack");
   FineArgs a = fine_args(ctx, ctx->ws_f, ctx->tab_f, n, batch, ctx->p.dt_fine, t0);
   if (full_io) {
@@ -890,7 +906,7 @@ kd_status kd_fine_batched(kd_ctx* ctx, const void* b_in, void* b_out, const doub
   if ((s = with_phases(ctx, ctx->ws_f, a, nsteps)) != KD_OK) return s;
   LaunchProbe pr = probe_of(ctx);
   if (nsteps > 0)
-    KD_LAUNCH(run_fine(ctx, 0, pf, a, nsteps, true, false, ctx->prof ? &pr : nullptr), "fine steps");
+    KD_LAUNCH(run_fine(ctx, 0, pf, a, nsteps, true, false, ctx->prof ? &pr : nullptr, nullptr, &plan), "fine steps");
   if (full_io)
     KD_LAUNCH(zero_outside_kept(pf, b_out, batch, n, ctx->st), "zero fill");
   else
@@ -900,7 +916,11 @@ kd_status kd_fine_batched(kd_ctx* ctx, const void* b_in, void* b_out, const doub
 
 kd_status kd_fine_batched_kept(kd_ctx* ctx, const void* c_in, void* c_out, const double* t0, int nsteps,
                                int batch) {
-  if (!ctx) return KD_EINVAL;
+  return ctx ? fine_kept(ctx, c_in, c_out, t0, nsteps, batch, call_plan(ctx, batch)) : KD_EINVAL;
+}
+
+static kd_status fine_kept(kd_ctx* ctx, const void* c_in, void* c_out, const double* t0, int nsteps, int batch,
+                           const FinePlan& plan) {
   if (!c_in || !c_out || !t0) return fail(ctx, KD_EINVAL, "kd_fine_batched_kept: NULL buffer");
   if (batch < 0 || nsteps < 0) return fail(ctx, KD_EINVAL, "kd_fine_batched_kept: negative batch or nsteps");
   const int n = ctx->p.n, pf = ctx->p.prec_fine;
@@ -926,7 +946,7 @@ kd_status kd_fine_batched_kept(kd_ctx* ctx, const void* c_in, void* c_out, const
   a.X = c_out;
   if ((s = with_phases(ctx, ctx->ws_f, a, nsteps)) != KD_OK) return s;
   LaunchProbe pr = probe_of(ctx);
-  KD_LAUNCH(run_fine(ctx, 0, pf, a, nsteps, true, false, ctx->prof ? &pr : nullptr), "fine steps");
+  KD_LAUNCH(run_fine(ctx, 0, pf, a, nsteps, true, false, ctx->prof ? &pr : nullptr, nullptr, &plan), "fine steps");
   return KD_OK;
 }
 
@@ -965,6 +985,7 @@ static kd_status host_chunks(kd_ctx* ctx, const void* h_in, void* h_out, const d
   // events per slot q: hev[q] input copied in, hev[2 + q] computed, hev[4 + q] output copied out
   KD_CUDA(cudaMemcpyAsync(ctx->hio_t0, t0, (size_t)batch * 8, cudaMemcpyHostToDevice, ctx->st), "times");
   for (int q = 2; q < 6; ++q) KD_CUDA(cudaEventRecord(ctx->hev[q], ctx->st), "event");
+  const FinePlan steps = call_plan(ctx, batch);
   int f0 = 0;
   for (int c = 0; c < (int)plan.size(); f0 += plan[c], ++c) {
     const int q = c & 1, nb = plan[c];
@@ -976,7 +997,7 @@ static kd_status host_chunks(kd_ctx* ctx, const void* h_in, void* h_out, const d
     // compute after the copy in, into an output slot that chunk c - 2 has left
     KD_CUDA(cudaStreamWaitEvent(ctx->st, ctx->hev[q], 0), "wait");
     KD_CUDA(cudaStreamWaitEvent(ctx->st, ctx->hev[4 + q], 0), "wait");
-    if ((s = kd_fine_batched(ctx, din, dout, ctx->hio_t0 + f0, nsteps, nb)) != KD_OK) return s;
+    if ((s = fine_full(ctx, din, dout, ctx->hio_t0 + f0, nsteps, nb, steps)) != KD_OK) return s;
     KD_CUDA(cudaEventRecord(ctx->hev[2 + q], ctx->st), "event");
     KD_CUDA(cudaStreamWaitEvent(ctx->st_d2h, ctx->hev[2 + q], 0), "wait");
     KD_CUDA(cudaMemcpyAsync((char*)h_out + f0 * fb, dout, nb * fb, cudaMemcpyDeviceToHost, ctx->st_d2h), "copy out");
@@ -993,6 +1014,7 @@ static kd_status host_chunks_kept(kd_ctx* ctx, const void* h_in, void* h_out, co
   // events per slot q: hev[q] copied in, hev[4 + q] computed, hev[8 + q] copied out
   KD_CUDA(cudaMemcpyAsync(ctx->hio_t0, t0, (size_t)batch * 8, cudaMemcpyHostToDevice, ctx->st), "times");
   for (int q = 0; q < 4; ++q) KD_CUDA(cudaEventRecord(ctx->hev[8 + q], ctx->st), "event");
+  const FinePlan steps = call_plan(ctx, batch);
   int f0 = 0;
   for (int c = 0; c < (int)plan.size(); f0 += plan[c], ++c) {
     const int q = c & 3, nb = plan[c];
@@ -1002,7 +1024,7 @@ static kd_status host_chunks_kept(kd_ctx* ctx, const void* h_in, void* h_out, co
     KD_CUDA(cudaMemcpyAsync(slot, (const char*)h_in + f0 * fb, nb * fb, cudaMemcpyHostToDevice, ctx->st_h2d), "copy in");
     KD_CUDA(cudaEventRecord(ctx->hev[q], ctx->st_h2d), "event");
     KD_CUDA(cudaStreamWaitEvent(ctx->st, ctx->hev[q], 0), "wait");
-    if ((s = kd_fine_batched_kept(ctx, slot, slot, ctx->hio_t0 + f0, nsteps, nb)) != KD_OK) return s;
+    if ((s = fine_kept(ctx, slot, slot, ctx->hio_t0 + f0, nsteps, nb, steps)) != KD_OK) return s;
     KD_CUDA(cudaEventRecord(ctx->hev[4 + q], ctx->st), "event");
     KD_CUDA(cudaStreamWaitEvent(ctx->st_d2h, ctx->hev[4 + q], 0), "wait");
     KD_CUDA(cudaMemcpyAsync((char*)h_out + f0 * fb, slot, nb * fb, cudaMemcpyDeviceToHost, ctx->st_d2h), "copy out");

@@ -184,10 +184,11 @@ extern "C" kd_status kd_growth_arnoldi(kd_ctx* ctx, const double* b0, double t0,
   KD_LAUNCH(full_to_compact(KD_C128, ctx->full_tmp, KD_C128, ar.V, 1, n, ctx->st), "pack");
 
   // w = M v (FP64 in and out; the propagator in the context's fine precision)
+  const FinePlan plan = call_plan(ctx, 1);
   auto apply = [&](const double2* v, double2* w) -> kd_status {
     if (conv) return conv_fine(ctx, (const double*)v, (double*)w, 1, S, dt, tdev);
     KD_LAUNCH(compact_resample(KD_C128, v, n, pf, ctx->ws_f.X, n, 1, ctx->st), "to fine precision");
-    KD_LAUNCH(run_fine(ctx, 0, pf, a, S, true, false), "fine steps");
+    KD_LAUNCH(run_fine(ctx, 0, pf, a, S, true, false, nullptr, nullptr, &plan), "fine steps");
     KD_LAUNCH(compact_resample(pf, ctx->ws_f.X, n, KD_C128, w, n, 1, ctx->st), "to FP64");
     return KD_OK;
   };

@@ -194,6 +194,10 @@ kd_status ensure_conv_tmp(kd_ctx* ctx, size_t bytes);
 kd_status conv_fine(kd_ctx* ctx, const double* in, double* out, long batch, int nsteps, double dt, const double* t0);
 // fine steps on grid g (0 fine, 1 coarse) with the context's plan for that grid
 int run_fine(kd_ctx* ctx, int g, int prec, const kd::FineArgs& a, int nsteps, bool prologue, bool store_last,
-             const kd::LaunchProbe* probe = nullptr, const int* active = nullptr);
+             const kd::LaunchProbe* probe = nullptr, const int* active = nullptr, const kd::FinePlan* plan = nullptr);
+// fine-grid plan of a call over `batch` fields in all: the context's, or where that is the
+// default one the default for a few fields (fine_few); a call that works in chunks asks for the
+// whole, so that its values do not depend on the chunks
+kd::FinePlan call_plan(const kd_ctx* ctx, long batch);
 
 }  // namespace kdi

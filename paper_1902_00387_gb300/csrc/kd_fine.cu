@@ -2,7 +2,8 @@
 // Parareal, Sec. 3 Eq. 8 and Sec. 4), all slices of a batch advanced by every launch.
 //
 // This file holds the flow-phase table and the dispatch to the kernel families
-// (kd_fine2.cuh for n <= 256, kd_fine3.cuh / kd_fine4.cuh for n = 512, 1024, instantiated
+// (kd_fused.cuh: the persistent step of n <= 286;
+// kd_fine2.cuh for n <= 256, kd_fine3.cuh / kd_fine4.cuh for n = 512, 1024, instantiated
 // per precision and grid in kd_fine2_*.cu / kd_fine3_*.cu; the mixed-radix kernels of
 // kd_fine_mr.cuh for n = 96, 160, 192 in kd_fine_mr.cu).  One right-hand-side
 // evaluation nabla_k x (u x b) followed by one IMEX stage is two kernels:
@@ -82,18 +83,20 @@ int launch_phases(int prec, const FineArgs& a, int nsteps, cudaStream_t st) {
 }
 
 template <typename T>
-static cudaError_t prepare_all() {
-  cudaError_t e;
-  if ((e = fine2_prep<T, 16>()) != cudaSuccess) return e;
-  if ((e = fine2_prep<T, 32>()) != cudaSuccess) return e;
-  if ((e = fine2_prep<T, 64>()) != cudaSuccess) return e;
-  if ((e = fine2_prep<T, 128>()) != cudaSuccess) return e;
-  if ((e = fine2_prep<T, 256>()) != cudaSuccess) return e;
-  if ((e = fine3_prep<T, 512>()) != cudaSuccess) return e;
-  return fine3_prep<T, 1024>();
+static cudaError_t prepare_T(int n) {
+  const int m = n ? fine_fft_grid(n) : 0;   // 0: every side
+  cudaError_t e = fused_prepare(sizeof(T) == 4 ? 0 : 1, n ? n / 3 : 0);
+  if (e == cudaSuccess && (!m || m == 16)) e = fine2_prep<T, 16>();
+  if (e == cudaSuccess && (!m || m == 32)) e = fine2_prep<T, 32>();
+  if (e == cudaSuccess && (!m || m == 64)) e = fine2_prep<T, 64>();
+  if (e == cudaSuccess && (!m || m == 128)) e = fine2_prep<T, 128>();
+  if (e == cudaSuccess && (!m || m == 256)) e = fine2_prep<T, 256>();
+  if (e == cudaSuccess && (!m || m == 512)) e = fine3_prep<T, 512>();
+  if (e == cudaSuccess && (!m || m == 1024)) e = fine3_prep<T, 1024>();
+  return e;
 }
 
-cudaError_t fine_prepare(int prec) { return prec == 0 ? prepare_all<float>() : prepare_all<double>(); }
+cudaError_t fine_prepare(int prec, int n) { return prec == 0 ? prepare_T<float>(n) : prepare_T<double>(n); }
 
 template <typename T>
 static bool variants_T(int n, int* ncol, int* nrow) {
@@ -113,11 +116,16 @@ static bool variants_T(int n, int* ncol, int* nrow) {
   return false;
 }
 
-FinePlan fine_default_plan(int n, int prec) {
-  if (fine_fft_grid(n) == 1024 && prec == 0) return fine3_default_plan<float, 1024>();
-  if (fine_fft_grid(n) == 512 && prec == 0) return fine3_default_plan<float, 512>();
-  if (fine_fft_grid(n) == 256 && prec == 0) return fine2_default_plan<float, 256>();
-  if (fine_fft_grid(n) == 128 && prec == 0) return fine2_default_plan<float, 128>();
+FinePlan fine_default_plan(int n, int prec, bool few) {
+  if (fine_fft_grid(n) == 1024 && prec == 0) return fine3_default_plan<float, 1024>(few);
+  if (fine_fft_grid(n) == 512 && prec == 0) return fine3_default_plan<float, 512>(few);
+  if (prec == 0) switch (n) {
+      case 16: return fine2_default_plan<float, 16>(few);
+      case 32: return fine2_default_plan<float, 32>(few);
+      case 64: return fine2_default_plan<float, 64>(few);
+      case 128: return fine2_default_plan<float, 128>(few);
+      case 256: return fine2_default_plan<float, 256>(few);
+    }
   return FinePlan();
 }
 
@@ -130,8 +138,20 @@ bool fine_variants(int n, int prec, int* ncol, int* nrow) {
   return prec == 0 ? variants_T<float>(m, ncol, nrow) : variants_T<double>(m, ncol, nrow);
 }
 
+// Whether a call goes to the persistent fused step: RK443 from the state to the state on a kept
+// set it covers; in complex128 and on the mixed-radix sides always (they have one plan), but for
+// the complex128 side 256, whose 256-point kernels are faster for a batch (32 fields: 4.8 ms a
+// step against 5.7; FP64 arithmetic bounds both); on the complex64 power-of-two sides with the
+// plan that selects it.
+static bool takes_fused(int prec, const FineArgs& a, const StepCfg& cfg) {
+  if (!fused_covers(a.K, a.scheme) || !cfg.prologue || cfg.store_last) return false;
+  if (fine_mr_side(a.n)) return true;
+  return prec != 0 ? a.n != 256 : cfg.plan.col == fused_col(a.n);
+}
+
 template <typename T>
 static int run_T(const FineArgs& a, const StepCfg& cfg) {
+  if (takes_fused(sizeof(T) == 4 ? 0 : 1, a, cfg)) return fused_run(sizeof(T) == 4 ? 0 : 1, a, cfg);
   switch (a.n) {
     case 16: return fine2_run<T, 16>(a, cfg);
     case 32: return fine2_run<T, 32>(a, cfg);

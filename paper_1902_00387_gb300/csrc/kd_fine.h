@@ -14,8 +14,8 @@ struct LaunchProbe {
 
 // Launch plan of the fine kernels: index of the column-kernel and row-kernel variant
 // (tile shape, stage-update style) among those instantiated for the grid and precision;
-// {0, 0} is the default ({6, 7} on the complex64 grid n = 1024, {5, 9} at n = 512 and
-// {0, 9} at n = 256, {1, 9} at n = 128, fine_default_plan).
+// {0, 0} is the default in complex128 and on the mixed-radix sides; complex64: {6, 7} at
+// n = 1024, {5, 9} at n = 512, {fused_col(n), 0} at n <= 256 (fine_default_plan).
 // Chosen per (n, precision, batch) by the autotuner.
 struct FinePlan {
   int col = 0;
@@ -37,7 +37,8 @@ struct StepCfg {
 };
 
 // ---- kd_fine.cu
-cudaError_t fine_prepare(int prec);
+// set the shared-memory limits of the kernels that grids of side n use (n = 0: of all kernels)
+cudaError_t fine_prepare(int prec, int n);
 // bytes of the flow-phase table FineArgs::phases for `batch` fields and `nsteps` steps
 size_t phase_table_bytes(int prec, long batch, int nsteps);
 // fill FineArgs::phases (Galloway-Proctor, or any batch with per-slice parameters);
@@ -45,8 +46,11 @@ size_t phase_table_bytes(int prec, long batch, int nsteps);
 int launch_phases(int prec, const FineArgs& a, int nsteps, cudaStream_t st);
 // number of column / row variants instantiated for (fine_fft_grid(n), prec); false if none
 bool fine_variants(int n, int prec, int* ncol, int* nrow);
-// launch plan of a context before any autotuning or kd_set_plan
-FinePlan fine_default_plan(int n, int prec);
+// launch plan of a context before any autotuning or kd_set_plan; few: for calls of at most
+// fine_few(n) fields (and for the coarse grid, whose serial sweep steps one at a time), which
+// leave most of the GPU idle in the default's larger blocks
+FinePlan fine_default_plan(int n, int prec, bool few = false);
+constexpr int fine_few(int n, int prec) { return prec != 0 ? 0 : (n == 256 ? 6 : (n == 512 ? 3 : 0)); }
 // Row variant of the warp-transform row kernel of the complex64 n = 1024 grid
 constexpr int kRow4Variant = 7;
 // whether the plan's kernels read the first step's state from FineArgs::x_in_full and
@@ -60,6 +64,15 @@ int fine_run(int prec, const FineArgs& a, const StepCfg& cfg);
 // the same with the default plan and every field taking every step
 int fine_launch_steps(int prec, const FineArgs& a, int nsteps, bool prologue, bool store_last,
                       cudaStream_t st, const LaunchProbe* probe = nullptr);
+
+// ---- kd_fused.cu: persistent fused step (kept sets K <= 95, i.e. n <= 286; RK443)
+bool fused_covers(int K, int scheme);
+cudaError_t fused_prepare(int prec, int K);   // the kernel of the kept set K (0: all)
+// Enqueue cfg.nsteps steps from a.X to a.X (a.phases filled); returns the kernels launched,
+// negative on failure.  Needs a prologue call that keeps no mixed field.
+int fused_run(int prec, const FineArgs& a, const StepCfg& cfg);
+// column variant of the complex64 sides 16..256 that selects it
+constexpr int fused_col(int n) { return n == 128 ? 4 : (n == 256 ? 6 : (n == 16 ? 3 : 4)); }
 
 // ---- kd_fine_mr.cu: grid sides 32 R that are not powers of two (96, 160, 192)
 bool fine_mr_side(int n);
@@ -92,7 +105,7 @@ cudaError_t fine2_prep();
 template <typename T, int N>
 void fine2_variants(int* ncol, int* nrow);
 template <typename T, int N>
-FinePlan fine2_default_plan();
+FinePlan fine2_default_plan(bool few);
 template <typename T, int N>
 int fine3_run(const FineArgs& a, const StepCfg& cfg);
 template <typename T, int N>
@@ -100,7 +113,7 @@ cudaError_t fine3_prep();
 template <typename T, int N>
 void fine3_variants(int* ncol, int* nrow);
 template <typename T, int N>
-FinePlan fine3_default_plan();
+FinePlan fine3_default_plan(bool few);
 
 // ---- kd_ops.cu (layout conversions, Parareal update, norms)
 // full [batch][3][n][n] (precision pin) -> compact [batch][3][P][P] (precision pout)

@@ -2,7 +2,8 @@
 // step loop (kd_fine.h: fine_run).  Included by the instantiation units kd_fine2_*.cu
 // and kd_fine3_*.cu.
 //
-// complex64 variants (complex128 has variant 0 only):
+// complex64 variants (complex128 has variant 0 only: RK443 on n <= 286, n = 256 aside, with the
+// fused step of kd_fused.cu, the rest with the first kernels below):
 //   n <= 256  column: 0, 1 = four-step kernels with XT0, XT0/2 columns per block;
 //                     2 = component-split four-step kernel (one component per thread);
 //                     3 = three-pass kernel with 8 values per thread (n = 128, 256)
@@ -11,11 +12,13 @@
 //                     6, 7 = three-pass, 8 values per thread, staged | registers (n = 128, 256)
 //             both:   the next variant = the warp-owned mixed-radix kernels of kd_fine_mr.cuh
 //                     (one warp per column / row with its three components; n = 32 .. 256);
-//                     at n = 256 the last = the 256-point warp-transform kernels of
-//                     kd_fine5.cuh (the row kernel for RK443)
+//                     at n = 256 and 128 the next = the warp-transform kernels of kd_fine5.cuh
+//                     (the row kernel for RK443)
+//             column: 4 at n = 128, the last at the other sides = the persistent fused step of
+//                     kd_fused.cu (the default; fused_col)
 //   n >= 512  column: 0, 1 = three-pass, 16 values per thread, XT0, XT0/2 columns;
 //                     2 = persistent prefetching kernel; 3 = component-split kernel;
-//                     4 = 8 values per thread (n = 512); 5 = 512-point warp transforms,
+//                     4 = 8 values per thread (n = 512); 5, 6 = 512-point warp transforms,
 //                     one warp per column (kd_fine5.cuh; n = 512)
 //             row:    0..3 = three-pass, 16 values, (RT0 | RT0/2) x (staged | registers);
 //                     4 = persistent prefetching kernel (in registers);
@@ -35,7 +38,6 @@
 #include "kd_fine2c.cuh"
 #include "kd_fine3.cuh"
 #include "kd_fine3c.cuh"
-#include "kd_fine2f.cuh"
 #include "kd_fine4.cuh"
 #include "kd_fine5.cuh"
 #include "kd_narrow.cuh"
@@ -66,8 +68,6 @@ static void launch_k(void (*k)(KArgs...), unsigned grid, unsigned block, size_t 
 template <typename T, int R>
 struct FineMrSet {
   static constexpr int N = 32 * R;
-  static constexpr bool FUSED = false;
-  static constexpr int kFusedCol = -1;
   static constexpr bool narrow(int, int, int) { return false; }
   static constexpr unsigned BLOCK = 32 * kMrWarps;
   static int ncol() { return 1; }
@@ -223,16 +223,63 @@ struct ShapesC {
   static constexpr int RT0 = 8, RT1 = 4;
 };
 
+// Kernels on N = 3n/4 points (kd_narrow.cuh): column kernel with kNarrowGroups groups a
+// block, one block per SM; row kernel with as many blocks per SM as fit.
+constexpr int kNarrowVariant = 100, kNarrowGroups = 3;
+
+template <int N>
+static void launch_coln(const FineArgs& a, int s, int j, cudaStream_t st, bool pdl) {
+  using C = ColN<N, kNarrowGroups>;
+  const long groups = (long)a.batch * (N / C::XG);
+  launch_k(coln_kernel<N, kNarrowGroups>, persistent_grid(groups), C::BLOCK, C::smem, st, pdl, a, s, j);
+}
+
+template <int N, int MODE>
+static void launch_rown_mode(const FineArgs& a, int store, cudaStream_t st, bool pdl) {
+  using G = RowN<N, MODE>;
+  const long blocks = ((long)a.batch * a.P + G::W::C - 1) / G::W::C;
+  const long cap = (long)persistent_grid(1L << 30) * G::MINB;
+  launch_k(rown_kernel<N, MODE>, (unsigned)(blocks < cap ? blocks : cap), G::BLOCK, G::smem, st, pdl, a, store);
+}
+
+template <int N>
+static void launch_rown(const FineArgs& a, int mode, int store, cudaStream_t st, bool pdl) {
+  switch (mode) {
+    case 0: return launch_rown_mode<N, 0>(a, store, st, pdl);
+    case 1: return launch_rown_mode<N, 1>(a, store, st, pdl);
+    case 2: return launch_rown_mode<N, 2>(a, store, st, pdl);
+    case 3: return launch_rown_mode<N, 3>(a, store, st, pdl);
+    default: return launch_rown_mode<N, 4>(a, store, st, pdl);
+  }
+}
+
+template <int N, int MODE>
+static cudaError_t prepare_rown() {
+  return cudaFuncSetAttribute(rown_kernel<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)RowN<N, MODE>::smem);
+}
+
+template <int N>
+static cudaError_t prepare_narrow() {
+  cudaError_t e = cudaFuncSetAttribute(coln_kernel<N, kNarrowGroups>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)ColN<N, kNarrowGroups>::smem);
+  if (e == cudaSuccess) e = prepare_rown<N, 0>();
+  if (e == cudaSuccess) e = prepare_rown<N, 1>();
+  if (e == cudaSuccess) e = prepare_rown<N, 2>();
+  if (e == cudaSuccess) e = prepare_rown<N, 3>();
+  if (e == cudaSuccess) e = prepare_rown<N, 4>();
+  return e;
+}
+
 template <typename T, int N>
 struct Fine2Set {
   using Sh = Shapes2<T, N>;
   using ShC = ShapesC<N>;
   static constexpr bool WIDE = sizeof(T) == 4;
   static constexpr bool R8 = WIDE && (N == 128 || N == 256);
-  // FP32 n = 128: column variant 4 is the persistent 2-block fused step (the row
-  // variant does not apply)
-  static constexpr bool FUSED = WIDE && N == 128;
-  static constexpr int kFusedCol = 4;
+  // one column variant of every complex64 side is the persistent fused step (kd_fused.cu, taken
+  // before these kernels are asked; the row variant does not apply): fused_col(N); the calls
+  // it does not cover run on column variant 0
   static constexpr bool narrow(int, int, int) { return false; }
   // the warp-owned mixed-radix kernels (FineMrSet) as a further column / row variant of
   // the sides 32 R, complex64 (complex128 keeps one plan: the serial fine run, tuned for
@@ -241,17 +288,19 @@ struct Fine2Set {
   static constexpr bool MR = WIDE && N % 32 == 0;
   // complex64 n = 256 and 128: the warp-transform kernels (kd_fine5.cuh) after that
   static constexpr bool WT = WIDE && (N == 256 || N == 128);
-  static int ncol0() { return WIDE ? (R8 ? (FUSED ? 5 : 4) : 3) : 1; }
+  static int ncol0() { return WIDE ? (R8 ? (N == 128 ? 5 : 4) : 3) : 1; }
   static int nrow0() { return WIDE ? (R8 ? 8 : 6) : 1; }
-  static int ncol() { return ncol0() + (MR ? 1 : 0) + (WT ? 1 : 0); }
+  static int ncol() { return ncol0() + (MR ? 1 : 0) + (WT ? 1 : 0) + (WIDE && N != 128 ? 1 : 0); }
   static int nrow() { return nrow0() + (MR ? 1 : 0) + (WT ? 1 : 0); }
-  // plan of a context that is not autotuned: the warp-transform row kernel with the
-  // four-step column kernel (n = 256) or its second tile shape (n = 128), measured fastest
-  // of the fixed plans
-  static FinePlan default_plan() {
+  // plan of a context that is not autotuned: the persistent fused step; for one field at a time
+  // (few) at n = 256 the warp-transform row kernel with the four-step column kernel, which spread
+  // a field over the whole GPU instead of 16 SMs (47 us a step against 59; 8 fields: 80 and 78)
+  static FinePlan default_plan(bool few) {
     FinePlan p;
-    if (WT) p.row = nrow0() + 1;
-    if (WT && N == 128) p.col = 1;
+    if (few && WT && N == 256)
+      p.row = nrow0() + 1;
+    else if (WIDE)
+      p.col = fused_col(N);
     return p;
   }
   static cudaError_t prepare() {
@@ -275,11 +324,6 @@ struct Fine2Set {
         return e;
       if ((e = cudaFuncSetAttribute(row2c_kernel<T, N, ShC::RT1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)Row2C<T, N, ShC::RT1>::smem)) != cudaSuccess)
-        return e;
-    }
-    if constexpr (FUSED) {
-      if ((e = cudaFuncSetAttribute(fused128_kernel<>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)Fused128::smem)) != cudaSuccess)
         return e;
     }
     if constexpr (R8) {
@@ -375,55 +419,6 @@ static cudaError_t prepare_row4() {
                               (int)G::smem);
 }
 
-// Kernels on N = 3n/4 points (kd_narrow.cuh): column kernel with kNarrowGroups groups a
-// block, one block per SM; row kernel with as many blocks per SM as fit.
-constexpr int kNarrowVariant = 100, kNarrowGroups = 3;
-
-template <int N>
-static void launch_coln(const FineArgs& a, int s, int j, cudaStream_t st, bool pdl) {
-  using C = ColN<N, kNarrowGroups>;
-  const long groups = (long)a.batch * (N / C::XG);
-  launch_k(coln_kernel<N, kNarrowGroups>, persistent_grid((groups + C::GR - 1) / C::GR), C::BLOCK, C::smem, st, pdl, a,
-           s, j);
-}
-
-template <int N, int MODE>
-static void launch_rown_mode(const FineArgs& a, int store, cudaStream_t st, bool pdl) {
-  using G = RowN<N, MODE>;
-  const long blocks = ((long)a.batch * a.P + G::W::C - 1) / G::W::C;
-  const long cap = (long)persistent_grid(1L << 30) * G::MINB;
-  launch_k(rown_kernel<N, MODE>, (unsigned)(blocks < cap ? blocks : cap), G::BLOCK, G::smem, st, pdl, a, store);
-}
-
-template <int N>
-static void launch_rown(const FineArgs& a, int mode, int store, cudaStream_t st, bool pdl) {
-  switch (mode) {
-    case 0: return launch_rown_mode<N, 0>(a, store, st, pdl);
-    case 1: return launch_rown_mode<N, 1>(a, store, st, pdl);
-    case 2: return launch_rown_mode<N, 2>(a, store, st, pdl);
-    case 3: return launch_rown_mode<N, 3>(a, store, st, pdl);
-    default: return launch_rown_mode<N, 4>(a, store, st, pdl);
-  }
-}
-
-template <int N, int MODE>
-static cudaError_t prepare_rown() {
-  return cudaFuncSetAttribute(rown_kernel<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)RowN<N, MODE>::smem);
-}
-
-template <int N>
-static cudaError_t prepare_narrow() {
-  cudaError_t e = cudaFuncSetAttribute(coln_kernel<N, kNarrowGroups>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)ColN<N, kNarrowGroups>::smem);
-  if (e == cudaSuccess) e = prepare_rown<N, 0>();
-  if (e == cudaSuccess) e = prepare_rown<N, 1>();
-  if (e == cudaSuccess) e = prepare_rown<N, 2>();
-  if (e == cudaSuccess) e = prepare_rown<N, 3>();
-  if (e == cudaSuccess) e = prepare_rown<N, 4>();
-  return e;
-}
-
 template <typename T, int N>
 struct Fine3Set {
   using Sh = Shapes3<T, N>;
@@ -434,22 +429,22 @@ struct Fine3Set {
   // n = 512: column variant 5 and row variant 9 are the 512-point warp-transform kernels
   static constexpr int kC512Col = 5, kC512Row = 9;
   static constexpr int XTC = Sh::XT0, RTC0 = Sh::RT0, RTC1 = Sh::RT0 / 2;
-  static constexpr bool FUSED = false;   // no persistent fused step at these sizes
-  static constexpr int kFusedCol = -1;
   // the pair of variants that steps on NN = 3n/4 points
   static constexpr int NN = N / 4 * 3;
   static constexpr bool narrow(int col, int row, int scheme) {
     return scheme == SCHEME_RK443 && ((W4 && col == kW6Col && row == kW4Row) || (R8 && col == kC512Col && row == kC512Row));
   }
-  static int ncol() { return WIDE ? (R8 ? 6 : (W4 ? 7 : 4)) : 1; }
-  // plan of a context that is not autotuned: the warp-transform kernels where they exist
-  static FinePlan default_plan() {
+  static int ncol() { return WIDE ? (R8 ? 7 : (W4 ? 7 : 4)) : 1; }
+  // plan of a context that is not autotuned: the 3n/4-point pairs; for up to three fields of
+  // 512^2 (few) the 512-point warp kernels, whose blocks are smaller (1, 2, 4 fields: 72, 80,
+  // 133 us a step against 88, 97, 132)
+  static FinePlan default_plan(bool few) {
     FinePlan p;
     if (W4) {
       p.col = kW6Col;
       p.row = kW4Row;
     } else if (R8) {
-      p.col = kC512Col;
+      p.col = few ? kC512Col + 1 : kC512Col;
       p.row = kC512Row;
     }
     return p;
@@ -533,7 +528,7 @@ struct Fine3Set {
     }
     if constexpr (R8) {
       if (v == 4) return launch_col3<T, N, Shapes8<N>::XT, 8>(a, s, j, st, pdl);
-      if (v == kC512Col) return launch_colw<N>(a, s, j, st, pdl);
+      if (v == kC512Col || v == kC512Col + 1) return launch_colw<N>(a, s, j, st, pdl);
     }
     if (WIDE && v == 2) {
       using C = Col3P<T, N, Sh::XT0>;
@@ -593,24 +588,9 @@ template <class Set>
 static int run_steps(const FineArgs& a0, const StepCfg& cfg) {
   const FinePlan pl = cfg.plan;
   int cv = pl.col >= 0 && pl.col < Set::ncol() ? pl.col : 0;
-  if constexpr (Set::FUSED) {
-    if (cv == Set::kFusedCol) cv = 0;   // (only for the calls the fused step does not cover)
-  }
   int rv = pl.row >= 0 && pl.row < Set::nrow() ? pl.row : 0;
   if (Set::narrow(cv, rv, a0.scheme)) cv = rv = kNarrowVariant;
   int launches = 0;
-  if constexpr (Set::FUSED) {
-    // the persistent fused step: every step of every field in one launch (RK443, from X,
-    // no mixed field kept at the end, all fields for all steps)
-    if (pl.col == Set::kFusedCol && cfg.prologue && !cfg.store_last && !cfg.active &&
-        a0.scheme == SCHEME_RK443 && cfg.nsteps > 0) {
-      FineArgs af = a0;
-      af.lo_valid = 0;
-      launch_k(fused128_kernel<>, (unsigned)(2 * a0.batch), Fused128::THREADS, Fused128::smem, cfg.st, cfg.pdl, af,
-               cfg.nsteps);
-      return 1;
-    }
-  }
   if (cfg.prologue) {
     Set::row(rv, a0, 4, 1, cfg.st, cfg.pdl);
     ++launches;
@@ -657,8 +637,8 @@ void fine2_variants(int* ncol, int* nrow) {
 }
 
 template <typename T, int N>
-FinePlan fine2_default_plan() {
-  return Fine2Set<T, N>::default_plan();
+FinePlan fine2_default_plan(bool few) {
+  return Fine2Set<T, N>::default_plan(few);
 }
 
 template <typename T, int N>
@@ -678,8 +658,8 @@ void fine3_variants(int* ncol, int* nrow) {
 }
 
 template <typename T, int N>
-FinePlan fine3_default_plan() {
-  return Fine3Set<T, N>::default_plan();
+FinePlan fine3_default_plan(bool few) {
+  return Fine3Set<T, N>::default_plan(few);
 }
 
 }  // namespace kd
@@ -689,9 +669,9 @@ FinePlan fine3_default_plan() {
   template int kd::fine2_run<T, N>(const kd::FineArgs&, const kd::StepCfg&); \
   template cudaError_t kd::fine2_prep<T, N>();                             \
   template void kd::fine2_variants<T, N>(int*, int*);                       \
-  template kd::FinePlan kd::fine2_default_plan<T, N>();
+  template kd::FinePlan kd::fine2_default_plan<T, N>(bool);
 #define KD_FINE3_INSTANTIATE(T, N)                                        \
   template int kd::fine3_run<T, N>(const kd::FineArgs&, const kd::StepCfg&); \
   template cudaError_t kd::fine3_prep<T, N>();                             \
   template void kd::fine3_variants<T, N>(int*, int*);              \
-  template kd::FinePlan kd::fine3_default_plan<T, N>();
+  template kd::FinePlan kd::fine3_default_plan<T, N>(bool);

@@ -102,6 +102,7 @@ extern "C" kd_status kd_growth_power(kd_ctx* ctx, const double* b0, double t0, d
   KD_LAUNCH(normalise(pf, X, len, n0, ctx->st), "normalise");
   FineArgs a = fine_args(ctx, ctx->ws_f, ctx->tab_f, n, 1, dt, tdev);
   if ((s = with_phases(ctx, ctx->ws_f, a, S)) != KD_OK) return s;
+  const FinePlan plan = call_plan(ctx, 1);
   double prev = NAN, cur = NAN;
   int it = 0;
   for (it = 1; it <= max_iter; ++it) {
@@ -109,7 +110,7 @@ extern "C" kd_status kd_growth_power(kd_ctx* ctx, const double* b0, double t0, d
     if (conv) {
       if ((s = conv_fine(ctx, (const double*)X, (double*)X, 1, S, dt, tdev)) != KD_OK) return s;
     } else {
-      KD_LAUNCH(run_fine(ctx, 0, pf, a, S, true, false), "fine steps");
+      KD_LAUNCH(run_fine(ctx, 0, pf, a, S, true, false, nullptr, nullptr, &plan), "fine steps");
     }
     KD_LAUNCH(norm2(pf, X, len, ctx->partials, n1, ctx->st), "norm");
     KD_CUDA(cudaMemcpyAsync(ctx->host_scal, n0, 16, cudaMemcpyDeviceToHost, ctx->st), "norm copy");

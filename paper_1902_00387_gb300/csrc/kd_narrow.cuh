@@ -82,7 +82,8 @@ __global__ void __launch_bounds__(ColN<N, GR>::BLOCK, 1) coln_kernel(FineArgs a,
   }
   __syncthreads();
   const long groups = (long)a.batch * GPF;
-  const long first = (long)blockIdx.x * GR + grp, stride = (long)gridDim.x * GR;
+  // neighbouring groups on different SMs, so that a few fields use all of them
+  const long first = blockIdx.x + (long)grp * gridDim.x, stride = (long)gridDim.x * GR;
   const long mine = groups > first ? (groups - 1 - first) / stride + 1 : 0;
   const cx<float>* M = (const cx<float>*)a.M;
   cx<float>* Wo = (cx<float>*)a.W;

@@ -111,7 +111,7 @@ extern "C" kd_status kd_fine_batched_static(const kd_params* p, const void* b_in
       g_prepared[dev][0] = g_prepared[dev][1] = false;
     }
     if (!g_prepared[dev][prec]) {
-      cudaError_t e = fine_prepare(prec);
+      cudaError_t e = fine_prepare(prec, 0);
       if (e != cudaSuccess) {
         fprintf(stderr, "kd_fine_batched_static: kernel set-up failed: %s\n", cudaGetErrorString(e));
         return KD_ECUDA;

@@ -278,6 +278,8 @@ kd_status kd_autotune(kd_ctx* ctx, int grid, int batch, int nsteps, const char* 
   FinePlan best_plan = saved;
   for (int c = 0; c < nc && s == KD_OK; ++c)
     for (int r = 0; r < nr && s == KD_OK; ++r) {
+      // the persistent fused step has no row kernel: one candidate
+      if (r > 0 && prec == KD_C64 && c == fused_col(n) && fused_covers(n / 3, a.scheme)) continue;
       ctx->plan[grid].col = c;
       ctx->plan[grid].row = r;
       if (fill_hash(prec, w.X, (long)batch * compact_len(n), 12345u, ctx->st) < 0 ||

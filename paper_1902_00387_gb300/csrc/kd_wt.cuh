@@ -73,6 +73,21 @@ __device__ __forceinline__ cx<T> wt_tw(int e) {       // w_N^e, 0 <= e < N
   return mk((T)g_w768.re[i], (T)g_w768.im[i]);
 }
 
+// a s + b on both components; complex64: one packed FP32x2 instruction (each component rounds
+// once, as a scalar fused multiply-add does).
+__device__ __forceinline__ cx<float> wt_fma(cx<float> a, float s, cx<float> b) {
+  const float2 r = __ffma2_rn(make_float2(a.x, a.y), make_float2(s, s), make_float2(b.x, b.y));
+  return mk(r.x, r.y);
+}
+__device__ __forceinline__ cx<double> wt_fma(cx<double> a, double s, cx<double> b) {
+  return mk(__fma_rn(a.x, s, b.x), __fma_rn(a.y, s, b.y));
+}
+__device__ __forceinline__ cx<float> wt_add(cx<float> a, cx<float> b) {
+  const float2 r = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+  return mk(r.x, r.y);
+}
+__device__ __forceinline__ cx<double> wt_add(cx<double> a, cx<double> b) { return a + b; }
+
 // 3-point DFT in place; (a, b, c) -> X[0], X[1], X[2].
 template <typename T, int DIR>
 __device__ __forceinline__ void wt_dft3(cx<T>& a, cx<T>& b, cx<T>& c) {
@@ -80,8 +95,8 @@ __device__ __forceinline__ void wt_dft3(cx<T>& a, cx<T>& b, cx<T>& c) {
   const cx<T> x0 = a;
   cx<T> t = b, d = c;
   bfly(t, d);                                          // t = b + c, d = b - c
-  a = x0 + t;
-  const cx<T> m = mk(x0.x - T(0.5) * t.x, x0.y - T(0.5) * t.y);
+  a = wt_add(x0, t);
+  const cx<T> m = wt_fma(t, T(-0.5), x0);
   b = mk(m.x - h * d.y, m.y + h * d.x);
   c = mk(m.x + h * d.y, m.y - h * d.x);
 }
@@ -140,8 +155,8 @@ struct WT {
   static __device__ __forceinline__ void table(cx<T>* s_tw) {
     for (int i = threadIdx.x; i < TAB; i += blockDim.x) s_tw[i] = wt_tw<N, T>(((i / V) * (i % V)) % N);
   }
-  // The spectral lane of lane l: lanes 24..31 repeat lane 23 (same addresses, same values), which
-  // costs no more than idling them and keeps the code free of divergence.
+  // The spectral lane of lane l: lanes 24..31 read and compute what lane 23 does (their values are
+  // not stored), which costs no more than idling them and keeps the code free of divergence.
   static __device__ __forceinline__ int slane(int l) { return l < 24 ? l : 23; }
   // transform and element of spectral register (round r, k) in spectral lane l
   static __device__ __forceinline__ int spec_c(int l, int r) { return CR == 1 ? r : 2 * r + (l >= V ? 1 : 0); }
@@ -167,7 +182,7 @@ struct WT {
       for (int m1 = 0; m1 < S; ++m1) {
         cx<T> y = s[r * S + bitrev<S>(m1)];
         if (m1 != 0) y = tw_mul<DIR>(y, s_tw[m1 * V + a]);
-        row[m1 * PITCH] = y;
+        if (l < 24) row[m1 * PITCH] = y;
       }
     }
     __syncwarp();

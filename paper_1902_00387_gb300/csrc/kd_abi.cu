@@ -1513,16 +1513,18 @@ struct TrainBufs {
   int* err = nullptr;   // set by the tensor-core GEMM if one of its bounded waits ran out
 };
 
-kd_status train_bufs(kd_ctx* ctx, TrainBufs& b, int mp, int nc) {
+// gathered: the pairs are copied (load_pairs) and the gradient product is used with its padding columns
+kd_status train_bufs(kd_ctx* ctx, TrainBufs& b, int mp, int nc, bool gathered = true) {
   kd_status s;
   const size_t m2 = 2 * (size_t)mp;
   const size_t ld = (nc + 7) & ~7;
-  if ((s = dalloc(ctx, (void**)&b.xp, m2 * nc * 4, "pairs x")) != KD_OK) return s;
-  if ((s = dalloc(ctx, (void**)&b.yp, m2 * nc * 4, "pairs y")) != KD_OK) return s;
+  if (gathered && (s = dalloc(ctx, (void**)&b.xp, m2 * nc * 4, "pairs x")) != KD_OK) return s;
+  if (gathered && (s = dalloc(ctx, (void**)&b.yp, m2 * nc * 4, "pairs y")) != KD_OK) return s;
   if ((s = dalloc(ctx, (void**)&b.yT, m2 * nc * 4, "y transposed")) != KD_OK) return s;
   if ((s = dalloc(ctx, (void**)&b.C1, 2 * (size_t)nc * m2 * 4, "forward product")) != KD_OK) return s;
   if ((s = dalloc(ctx, (void**)&b.C2, 2 * (size_t)nc * ld * 4, "gradient product")) != KD_OK) return s;
-  KD_CUDA(cudaMemsetAsync(b.C2, 0, 2 * (size_t)nc * ld * 4, ctx->st), "memset");   // padding columns stay 0
+  if (gathered)
+    KD_CUDA(cudaMemsetAsync(b.C2, 0, 2 * (size_t)nc * ld * 4, ctx->st), "memset");   // padding columns stay 0
   if ((s = dalloc(ctx, (void**)&b.Xs, m2 * ld * 2, "x operand")) != KD_OK) return s;
   if ((s = dalloc(ctx, (void**)&b.XtT, m2 * nc * 2, "x^T operand")) != KD_OK) return s;
   if ((s = dalloc(ctx, (void**)&b.A2, 2 * (size_t)nc * m2 * 2, "residual operand")) != KD_OK) return s;
@@ -1567,8 +1569,8 @@ kd_status load_pairs(kd_ctx* ctx, TrainBufs& b, const float* x, const float* y, 
                             ctx->st),
             "gather y");
   }
-  KD_LAUNCH(learned_pack_x(b.xp, mp, nc, (nc + 7) & ~7, b.Xs, b.XtT, ctx->st), "pack x");
-  KD_LAUNCH(learned_transpose_y(b.yp, mp, nc, b.yT, ctx->st), "transpose y");
+  KD_LAUNCH(learned_pack_x(b.xp, mp, mp, nc, (nc + 7) & ~7, b.Xs, b.XtT, ctx->st), "pack x");
+  KD_LAUNCH(learned_transpose_y(b.yp, mp, mp, nc, b.yT, ctx->st), "transpose y");
   return KD_OK;
 }
 
@@ -1813,30 +1815,18 @@ kd_status kd_learned_loss_grad(kd_ctx* ctx, const float* W, const float* W0, flo
   if (ctx->p.learned_modes <= 0 || !W || !x || !y || n <= 0 || !loss_out || !grad_out)
     return fail(ctx, KD_EINVAL, "kd_learned_loss_grad: bad arguments");
   const int P = ctx->cP, nc = 3 * P * P, ld = (nc + 7) & ~7;
-  const size_t wcount = (size_t)2 * nc * ld;
   const int mp = (int)roundup4(n);
-  std::vector<int> idx(n);
-  for (int i = 0; i < n; ++i) idx[i] = i;
   kd_status s;
   TrainBufs b;
-  float *Wp = nullptr, *W0p = nullptr, *gp = nullptr;
-  if ((s = train_bufs(ctx, b, mp, nc)) != KD_OK) return s;
-  // the caller's [2 nc][nc] matrices in the padded [2 nc][ld] layout
-  if ((s = dalloc(ctx, (void**)&Wp, wcount * 4, "weights")) != KD_OK) return s;
-  if ((s = dalloc(ctx, (void**)&W0p, wcount * 4, "centre")) != KD_OK) return s;
-  if ((s = dalloc(ctx, (void**)&gp, wcount * 4, "gradient")) != KD_OK) return s;
-  KD_CUDA(cudaMemsetAsync(Wp, 0, wcount * 4, ctx->st), "memset");
-  KD_CUDA(cudaMemsetAsync(W0p, 0, wcount * 4, ctx->st), "memset");
-  KD_CUDA(cudaMemcpy2DAsync(Wp, ld * 4, W, nc * 4, nc * 4, 2 * nc, cudaMemcpyDeviceToDevice, ctx->st), "repack");
-  if (W0)
-    KD_CUDA(cudaMemcpy2DAsync(W0p, ld * 4, W0, nc * 4, nc * 4, 2 * nc, cudaMemcpyDeviceToDevice, ctx->st), "repack");
-  if ((s = load_pairs(ctx, b, x, y, idx, mp, nc)) != KD_OK) return s;
-  KD_LAUNCH(f32_to_bf16(Wp, b.Wbf, (long)wcount, ctx->st), "bf16");
+  if ((s = train_bufs(ctx, b, mp, nc, false)) != KD_OK) return s;
+  // the operands are padded to mp pairs and ld columns; pairs and FP32 matrices are read as the caller holds them
+  KD_LAUNCH(learned_pack_x(x, n, mp, nc, ld, b.Xs, b.XtT, ctx->st), "pack x");
+  KD_LAUNCH(learned_transpose_y(y, n, mp, nc, b.yT, ctx->st), "transpose y");
+  KD_LAUNCH(learned_weights_bf16(W, 2 * nc, nc, ld, b.Wbf, ctx->st), "bf16");
   if ((s = forward_backward(ctx, b, mp, nc, ctx->scal + 8)) != KD_OK) return s;
-  KD_LAUNCH(learned_grad(Wp, W0p, b.C2, gp, (long)wcount, 2.f / n, weight_decay, ctx->st), "gradient");
-  KD_CUDA(cudaMemcpy2DAsync(grad_out, nc * 4, gp, ld * 4, nc * 4, 2 * nc, cudaMemcpyDeviceToDevice, ctx->st), "unpack");
-  const int nb = diff_norms(Wp, W0p, (long)wcount, ctx->partials, ctx->st);
-  if (nb < 0) return fail(ctx, KD_ECUDA, "norm launch failed");
+  const int nb = learned_grad_norm(W, W0, b.C2, ld, grad_out, 2 * nc, nc, 2.f / n, weight_decay, ctx->partials, ctx->st);
+  if (nb < 0) return fail(ctx, KD_ECUDA, "gradient launch failed");
+  ctx->launches += 1;
   KD_LAUNCH(sum_partials(ctx->partials, nb, ctx->scal + 10, ctx->st), "norm");
   double h[4];
   KD_CUDA(cudaMemcpyAsync(h, ctx->scal + 8, 32, cudaMemcpyDeviceToHost, ctx->st), "loss");
@@ -1844,9 +1834,6 @@ kd_status kd_learned_loss_grad(kd_ctx* ctx, const float* W, const float* W0, flo
   *loss_out = h[0] / n + weight_decay * h[2];
   if ((s = check_gemm(ctx, b)) != KD_OK) return s;
   free_train_bufs(ctx, b);
-  dfree(ctx, Wp);
-  dfree(ctx, W0p);
-  dfree(ctx, gp);
   return KD_OK;
 }
 

@@ -382,40 +382,72 @@ int gemm_bf16_tn(const __nv_bfloat16* A, const __nv_bfloat16* Bt, float* C, int 
 }
 
 // ---------------------------------------------------------------- training
-__global__ void k_pack_x(const float* x, int m, int nc, int ld, __nv_bfloat16* Xs, __nv_bfloat16* XtT, long total) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const long n = i / ld;
-    const int j = (int)(i - n * ld);
-    const bool in = j < nc;
-    const __nv_bfloat16 re = __float2bfloat16(in ? x[2 * (n * nc + j)] : 0.f);
-    const __nv_bfloat16 im = __float2bfloat16(in ? x[2 * (n * nc + j) + 1] : 0.f);
-    Xs[n * ld + j] = re;
-    Xs[(m + n) * ld + j] = im;
-    if (in) {
-      XtT[(long)j * 2 * m + n] = re;
-      XtT[(long)j * 2 * m + m + n] = im;
+// Operands of m pairs from the vectors x, y [rows][nc] (complex FP32; pairs rows..m-1 are zero).
+// Both kernels move 32 x 32 tiles (unknown x pair) through shared memory: reads run along the
+// unknowns and the transposed writes along the pairs, both in whole sectors.  x and y are a
+// caller's arrays: read as single floats, they need no more than their alignment.
+constexpr int PT = 32, PR = TB / PT;
+
+__global__ void __launch_bounds__(TB) k_pack_x(const float* x, int rows, int m, int nc, int ld, __nv_bfloat16* Xs,
+                                               __nv_bfloat16* XtT, long tiles) {
+  __shared__ __nv_bfloat162 tile[PT][PT + 1];
+  const int tj = (ld + PT - 1) / PT, c = threadIdx.x % PT, r = threadIdx.x / PT;
+  for (long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const int j0 = (int)(t % tj) * PT, n0 = (int)(t / tj) * PT;
+    for (int q = r; q < PT; q += PR) {
+      const int n = n0 + q, j = j0 + c;
+      const bool in = n < rows && j < nc;
+      const long e = 2 * ((long)n * nc + j);
+      const __nv_bfloat162 h = __floats2bfloat162_rn(in ? x[e] : 0.f, in ? x[e + 1] : 0.f);
+      tile[q][c] = h;
+      if (n < m && j < ld) {
+        Xs[(long)n * ld + j] = h.x;
+        Xs[(long)(m + n) * ld + j] = h.y;
+      }
     }
+    __syncthreads();
+    for (int q = r; q < PT; q += PR) {
+      const int n = n0 + c, j = j0 + q;
+      if (n < m && j < nc) {
+        const __nv_bfloat162 h = tile[c][q];
+        XtT[(long)j * 2 * m + n] = h.x;
+        XtT[(long)j * 2 * m + m + n] = h.y;
+      }
+    }
+    __syncthreads();
   }
 }
 
-int learned_pack_x(const float* x, int m, int nc, int ld, __nv_bfloat16* Xs, __nv_bfloat16* XtT, cudaStream_t st) {
-  const long total = (long)m * ld;
-  k_pack_x<<<grid1(total), TB, 0, st>>>(x, m, nc, ld, Xs, XtT, total);
+int learned_pack_x(const float* x, int rows, int m, int nc, int ld, __nv_bfloat16* Xs, __nv_bfloat16* XtT,
+                   cudaStream_t st) {
+  const long tiles = (long)((ld + PT - 1) / PT) * ((m + PT - 1) / PT);
+  k_pack_x<<<(unsigned)(tiles < 65535 ? tiles : 65535), TB, 0, st>>>(x, rows, m, nc, ld, Xs, XtT, tiles);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
-__global__ void k_transpose_y(const float* y, int m, int nc, float* yT, long total) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const long n = i / nc;
-    const int j = (int)(i - n * nc);
-    yT[2 * ((long)j * m + n)] = y[2 * i];
-    yT[2 * ((long)j * m + n) + 1] = y[2 * i + 1];
+__global__ void __launch_bounds__(TB) k_transpose_y(const float* y, int rows, int m, int nc, float2* yT, long tiles) {
+  __shared__ float2 tile[PT][PT + 1];
+  const int tj = (nc + PT - 1) / PT, c = threadIdx.x % PT, r = threadIdx.x / PT;
+  for (long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const int j0 = (int)(t % tj) * PT, n0 = (int)(t / tj) * PT;
+    for (int q = r; q < PT; q += PR) {
+      const int n = n0 + q, j = j0 + c;
+      const bool in = n < rows && j < nc;
+      const long e = 2 * ((long)n * nc + j);
+      tile[q][c] = make_float2(in ? y[e] : 0.f, in ? y[e + 1] : 0.f);
+    }
+    __syncthreads();
+    for (int q = r; q < PT; q += PR) {
+      const int n = n0 + c, j = j0 + q;
+      if (n < m && j < nc) yT[(long)j * m + n] = tile[c][q];
+    }
+    __syncthreads();
   }
 }
 
-int learned_transpose_y(const float* y, int m, int nc, float* yT, cudaStream_t st) {
-  const long total = (long)m * nc;
-  k_transpose_y<<<grid1(total), TB, 0, st>>>(y, m, nc, yT, total);
+int learned_transpose_y(const float* y, int rows, int m, int nc, float* yT, cudaStream_t st) {
+  const long tiles = (long)((nc + PT - 1) / PT) * ((m + PT - 1) / PT);
+  k_transpose_y<<<(unsigned)(tiles < 65535 ? tiles : 65535), TB, 0, st>>>(y, rows, m, nc, (float2*)yT, tiles);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
@@ -501,17 +533,68 @@ int learned_momentum(float* W, const float* W0, const float* C2, float* v, __nv_
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
-__global__ void k_grad(const float* W, const float* W0, const float* C2, float* grad, long count, float scale,
-                       float wd) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < count; i += (long)gridDim.x * blockDim.x) {
-    const float d0 = W0 ? W[i] - W0[i] : W[i];
-    grad[i] = scale * C2[i] + 2.f * wd * d0;
+// The gradient grad = scale C2 + 2 wd (W - W0) of a caller's unpadded [rows][nc] matrices (C2: row
+// stride ldc) and, in the same pass, per-block sums of |W - W0|^2 (partials[2 b], [2 b + 1] = 0).
+// Bound by HBM: four matrices cross it once (1.66 GB at nc = 7203).  With the gradient, its
+// unpacking and the norm in passes of their own over padded copies of W and W0, and those copies
+// allocated and filled by each call, a call with 256 pairs took 8.0 ms; it takes 2.1.  The norm is
+// summed as an unevaluated pair of floats a thread (differences, squares and sums with their
+// rounding errors, ~45 bits) and in FP64 across threads: an FP64 product and sum per element
+// would be bound by the few FP64 units.
+__global__ void __launch_bounds__(TB) k_grad_norm(const float* W, const float* W0, const float* C2, int ldc,
+                                                  float* grad, int rows, int nc, float scale, float wd,
+                                                  double* partials) {
+  float sum = 0.f, low = 0.f;
+  double far = 0.0;
+  const int chunks = (nc + TB - 1) / TB;
+  for (long t = blockIdx.x; t < (long)rows * chunks; t += gridDim.x) {
+    const int row = (int)(t / chunks), j = (int)(t - (long)row * chunks) * TB + threadIdx.x;
+    if (j >= nc) continue;
+    const long i = (long)row * nc + j;
+    const float w = W[i], w0 = W0 ? W0[i] : 0.f;
+    const float d = w - w0, bb = d - w;
+    const float dl = (w - (d - bb)) + (-w0 - bb);            // w - w0 = d + dl exactly
+    grad[i] = scale * C2[(long)row * ldc + j] + 2.f * wd * d;
+    const float p = __fmul_rn(d, d);
+    if (d == 0.f) continue;
+    if (!(p > 1e-24f && p < 1e30f)) {                        // no FP32 pair holds this square
+      const double e = (double)w - (double)w0;
+      far += e * e;
+      continue;
+    }
+    const float pl = __fmaf_rn(2.f * d, dl, __fmaf_rn(d, d, -p));   // (w - w0)^2 = p + pl
+    const float s = sum + p, sb = s - sum;
+    low += ((sum - (s - sb)) + (p - sb)) + pl;
+    sum = s;
+  }
+  block_sum2((double)sum + (double)low + far, 0.0, partials);
+}
+
+int learned_grad_norm(const float* W, const float* W0, const float* C2, int ldc, float* grad, int rows, int nc,
+                      float scale, float wd, double* partials, cudaStream_t st) {
+  const long total = (long)rows * ((nc + TB - 1) / TB);
+  const unsigned g = (unsigned)(total < 1024 ? total : 1024);   // the partials' capacity
+  k_grad_norm<<<g, TB, 0, st>>>(W, W0, C2, ldc, grad, rows, nc, scale, wd, partials);
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? -(int)e : (int)g;
+}
+
+// BF16 rows of ld columns (zero beyond nc) of an unpadded FP32 matrix [rows][nc]; a thread writes
+// two columns.
+__global__ void __launch_bounds__(TB) k_weights_bf16(const float* W, int rows, int nc, int ld, __nv_bfloat16* Wbf) {
+  const int half = ld / 2, chunks = (half + TB - 1) / TB;
+  for (long t = blockIdx.x; t < (long)rows * chunks; t += gridDim.x) {
+    const int row = (int)(t / chunks), q = (int)(t - (long)row * chunks) * TB + threadIdx.x;
+    if (q >= half) continue;
+    const float* w = W + (long)row * nc;
+    const float a = 2 * q < nc ? w[2 * q] : 0.f, b = 2 * q + 1 < nc ? w[2 * q + 1] : 0.f;
+    *(__nv_bfloat162*)(Wbf + (long)row * ld + 2 * q) = __floats2bfloat162_rn(a, b);
   }
 }
 
-int learned_grad(const float* W, const float* W0, const float* C2, float* grad, long count, float scale, float wd,
-                 cudaStream_t st) {
-  k_grad<<<grid1(count), TB, 0, st>>>(W, W0, C2, grad, count, scale, wd);
+int learned_weights_bf16(const float* W, int rows, int nc, int ld, __nv_bfloat16* Wbf, cudaStream_t st) {
+  const long total = (long)rows * ((ld / 2 + TB - 1) / TB);
+  k_weights_bf16<<<(unsigned)(total < 65535 ? total : 65535), TB, 0, st>>>(W, rows, nc, ld, Wbf);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 

@@ -49,9 +49,9 @@ int gemm_bf16_tn_tc(const __nv_bfloat16* A, const __nv_bfloat16* Bt, float* C, i
 // training helpers (m pairs, nc complex unknowns)
 // Xs[2m][ld]  rows n: Re x_n, rows m + n: Im x_n (zero beyond nc)  (forward B operand)
 // XtT[nc][2m] row j: (Re x_n[j])_n, (Im x_n[j])_n                    (gradient B operand)
-int learned_pack_x(const float* x, int m, int nc, int ld, __nv_bfloat16* Xs, __nv_bfloat16* XtT, cudaStream_t st);
+int learned_pack_x(const float* x, int rows, int m, int nc, int ld, __nv_bfloat16* Xs, __nv_bfloat16* XtT, cudaStream_t st);
 // yT[nc][m] complex FP32 from y[m][nc]
-int learned_transpose_y(const float* y, int m, int nc, float* yT, cudaStream_t st);
+int learned_transpose_y(const float* y, int rows, int m, int nc, float* yT, cudaStream_t st);
 // from C1[2nc][2m] = W_stack . Xs^T: residual R = W x_n - y_n, loss partials (per-block
 // sum of |R|^2 into partials), and the gradient A operand
 // A2[2nc][2m]: row j: (R_r, R_i), row nc + j: (R_i, -R_r)
@@ -66,9 +66,13 @@ int learned_adam(float* W, const float* W0, const float* C2, float* m1, float* v
 // heavy-ball step: g as above, v = mu v + g, W -= eta v, Wbf = bf16(W)
 int learned_momentum(float* W, const float* W0, const float* C2, float* v, __nv_bfloat16* Wbf, long count,
                      float scale, float wd, float eta, float mu, cudaStream_t st);
-// plain gradient (no update): grad = scale * C2 + 2 wd (W - W0)   (W0 may be NULL)
-int learned_grad(const float* W, const float* W0, const float* C2, float* grad, long count, float scale, float wd,
-                 cudaStream_t st);
+// plain gradient (no update) of unpadded [rows][nc] matrices: grad = scale * C2 + 2 wd (W - W0)
+// (C2 with row stride ldc; W0 may be NULL), and per-block sums of |W - W0|^2 into partials;
+// returns the block count
+int learned_grad_norm(const float* W, const float* W0, const float* C2, int ldc, float* grad, int rows, int nc,
+                      float scale, float wd, double* partials, cudaStream_t st);
+// Wbf [rows][ld] = bf16(W [rows][nc]), zero beyond nc (ld even)
+int learned_weights_bf16(const float* W, int rows, int nc, int ld, __nv_bfloat16* Wbf, cudaStream_t st);
 int f32_to_bf16(const float* x, __nv_bfloat16* y, long count, cudaStream_t st);
 // sum of `count` doubles in fixed order -> out[0]
 int sum_partials(const double* p, int count, double* out, cudaStream_t st);

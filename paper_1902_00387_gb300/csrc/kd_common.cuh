@@ -48,6 +48,9 @@ __host__ __device__ __forceinline__ cx<T> mul_i(cx<T> a) { return mk(-a.y, a.x);
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
+// the 128-byte line at p (global memory) into L2
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Flow identifiers (match include/kd.h).
 enum { FLOW_ROBERTS = 0, FLOW_GP = 1, FLOW_NONE = 2 };
 

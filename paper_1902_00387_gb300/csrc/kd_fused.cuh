@@ -239,15 +239,6 @@ __device__ __forceinline__ cx<T>& fused_at(cx<T>* p, unsigned o) {
   return *(cx<T>*)((char*)p + o);
 }
 
-// h / (1 + h) for h >= 0 (implicit_gain): in complex64 an approximate reciprocal and one
-// residual correction of the quotient (Markstein's step), which rounds it as the division does but
-// for rare last-bit cases, without the division's range checks (1 + h is never tiny or huge).
-__device__ __forceinline__ float fused_gain(float h) {
-  const float d = 1.f + h, r = __fdividef(1.f, d), q = h * r;
-  return __fmaf_rn(__fmaf_rn(-q, d, h), r, q);
-}
-__device__ __forceinline__ double fused_gain(double h) { return implicit_gain(h); }
-
 // One component of one IMEX RK443 stage (the expressions of stage_update, kd_stage.cuh): f =
 // F_c(X_j); r the arrays read: X (stage 0), R2 R3 R4 (1), R3 R4 (2), R4 X Xlo (3); o: where the
 // arrays written go: R2 R3 R4; R3 R4; R4; X Xlo; stored where `on`.  Returns X_{j+1}.

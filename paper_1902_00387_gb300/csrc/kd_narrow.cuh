@@ -6,8 +6,10 @@
 // component of C ky rows), both persistent.  What bounds them at 1024^2 x 256: the column
 // kernel the shared-memory data pipe (71% of its wavefronts by the counters; transposes,
 // twiddles, staging), the row kernel HBM (4.7 TB/s on its bytes) and the latency of its loads.
-// Measured per launch against the 1024-point kernels: column 2.30 ms (3.13), row 3.60 ms
-// (3.97), a step 25.1 ms (30.2); a step of 45 fields of 512^2 1.16 ms (1.38).  Two column groups
+// A step measured against the 1024-point kernels (column 3.13 ms, row 3.97 a launch): 23.0 ms
+// (30.2), the column kernel 2.30 a launch; a step of 45 fields of 512^2 1.02 ms (1.38).  With all
+// the stage arrays of a row staged in shared memory (three blocks an SM instead of five at stages
+// 1 and 3) and three accumulators stored by stage 0 the steps took 25.3 and 1.15 ms.  Two column groups
 // a block (8 warps, 255 registers) took 2.32 ms, so a third (12 warps, 168 registers, 160
 // bytes of spills) gains little; the components in rolled loops (38 instead of 92 KB of
 // code) 2.85 ms, for the register moves and the lost overlap.
@@ -182,17 +184,44 @@ __global__ void __launch_bounds__(ColN<N, GR>::BLOCK, 1) coln_kernel(FineArgs a,
 // A block of three warps owns C ky rows, one warp per component.  The forward transform's
 // kept values go to the warp's buffer in wavenumber order, where the curl reads the other
 // two components and the stage update runs over consecutive kx on all 32 lanes (22 slots),
-// with coalesced accesses of the stage arrays; those are copied to shared memory by cp.async
-// while the row is transformed.
+// with coalesced accesses of the stage arrays.  The first of them is copied to shared memory by
+// cp.async while the row is transformed (its place takes the new stage value), the others are
+// brought into L2 meanwhile and loaded by the update.
+//
+// Stage arrays: stage 0 stores its explicit term f0 alone (in R2's place) and stage 1 forms X1 and
+// the accumulators from X and f0 again, the same operations in the same order: a step moves 14
+// compact fields through HBM instead of 17 (X | f0; X f0 | R3 R4; R3 R4 | R4; R4 X Xlo | X Xlo).
+constexpr int rown_reads(int mode) { return mode == 3 ? 3 : (mode == 4 ? 0 : (mode == 0 ? 1 : 2)); }
+
+template <int MODE>
+__device__ __forceinline__ cx<float> rown_update(const StageCoef<float>& q, const StageArrays<float>& sa, long s,
+                                                 float g, float dl, const cx<float>* r, cx<float> f,
+                                                 cx<float>* xout) {
+  const float dt = q.dt;
+  if (MODE == 0) {
+    sa.R2[s] = f;
+    return implicit_solve(r[0] + f * (dt * 0.5f), g);
+  }
+  if (MODE == 1) {
+    const cx<float> x0 = r[0], f0 = r[1], x1 = implicit_solve(x0 + f0 * (dt * 0.5f), g);
+    const cx<float> r2 = x0 + f0 * (dt * float(11.0 / 18.0)) - x1 * (dl * float(1.0 / 6.0));
+    const cx<float> r3 = x0 + f0 * (dt * float(5.0 / 6.0)) + x1 * (dl * 0.5f);
+    const cx<float> r4 = f0 * (dt * 0.25f) - x1 * (dl * 1.5f);
+    const cx<float> a[3] = {r2, r3, r4};
+    return stage_update_1<1>(q, sa, s, g, dl, a, f, nullptr);
+  }
+  return stage_update_1<MODE>(q, sa, s, g, dl, r, f, xout);
+}
+
 template <int N, int MODE>
 struct RowN {
   using G = NarrowGrid<N>;
   using W = typename G::W;
   static constexpr int BLOCK = 96, P = G::P;
-  static constexpr int NPRE = row4_reads(MODE);
+  static constexpr int NPRE = rown_reads(MODE), NST = NPRE < 1 ? 0 : 1;   // arrays read, of them staged
   static constexpr int ELEMS = W::C * P, SLOTS = (ELEMS + 31) / 32;
   static_assert(ELEMS <= W::BUF, "the kept values fit the transpose buffer");
-  static constexpr int WSM = W::BUF + NPRE * SLOTS * 32;   // complex per warp
+  static constexpr int WSM = W::BUF + NST * SLOTS * 32;    // complex per warp
   static constexpr size_t smem = ((size_t)3 * WSM + W::TAB) * sizeof(cx<float>);
   static constexpr int FIT = (int)(233472 / (smem + 1024));
   static constexpr int MINB = FIT > 5 ? 5 : FIT;           // 5: 128 registers a thread
@@ -215,11 +244,11 @@ __global__ void __launch_bounds__(RowN<N, MODE>::BLOCK, RowN<N, MODE>::MINB) row
   W::table(s_tw);
   __syncthreads();
   const StageArrays<float> sa = stage_arrays<float>(a);
-  const cx<float>* src[3] = {MODE == 0 ? sa.X : (MODE == 1 ? sa.R2 : (MODE == 2 ? sa.R3 : sa.R4)),
-                             MODE == 1 ? sa.R3 : (MODE == 2 ? sa.R4 : sa.X), MODE == 1 ? sa.R4 : sa.Xlo};
-  // the array holding the state X among src (stages 0 and 3), read from the caller's layout
+  const cx<float>* src[3] = {MODE <= 1 ? sa.X : (MODE == 2 ? sa.R3 : sa.R4),
+                             MODE == 1 ? sa.R2 : (MODE == 2 ? sa.R4 : sa.X), sa.Xlo};
+  // the array holding the state X among src (stages 0, 1 and 3), read from the caller's layout
   // [batch][3][FULL][FULL] in the first step when x_in_full is set
-  constexpr int XSRC = MODE == 0 ? 0 : (MODE == 3 ? 1 : -1);
+  constexpr int XSRC = MODE <= 1 ? 0 : (MODE == 3 ? 1 : -1);
   const cx<float>* xin = (const cx<float>*)a.x_in_full;
   cx<float>* xout = MODE == 3 ? (cx<float>*)a.x_out_full : nullptr;
   const int npre = MODE == 3 && !sa.lo_valid ? 2 : NPRE;   // before the first step the low part is zero
@@ -257,18 +286,24 @@ __global__ void __launch_bounds__(RowN<N, MODE>::BLOCK, RowN<N, MODE>::MINB) row
         }
       }
     } else {
+      auto addr = [&](int t, int i, int j) {
+        return t == XSRC && xin ? xin + full_at(i, j) : src[t] + at(cb, i) + j;
+      };
 #pragma unroll
-      for (int t = 0; t < NPRE; ++t)
+      for (int q = 0; q < SLOTS; ++q) {
+        const int e = lane + 32 * q;
+        if (valid(e)) cp_async8(Q + e, addr(0, row_of(e), e - row_of(e) * P));
+      }
+      cp_async_commit();
+      // the other arrays into L2 meanwhile, a lane a 128-byte line
+#pragma unroll
+      for (int t = 1; t < NPRE; ++t)
         if (t < npre)
 #pragma unroll
-          for (int q = 0; q < SLOTS; ++q) {
-            const int e = lane + 32 * q;
-            if (valid(e)) {
-              const int i = row_of(e), j = e - i * P;
-              cp_async8(Q + t * SLOTS * 32 + e, t == XSRC && xin ? xin + full_at(i, j) : src[t] + at(cb, i) + j);
-            }
+          for (int q = 0; q < (ELEMS + 511) / 512; ++q) {
+            const int e = 16 * (lane + 32 * q);
+            if (valid(e)) prefetch_l2(addr(t, row_of(e), e - row_of(e) * P));
           }
-      cp_async_commit();
       const cx<float>* Wr = (const cx<float>*)a.W + at(mb, W::phys_c(lane)) + W::phys_m1(lane);
 #pragma unroll
       for (int p = 0; p < V; ++p) v[p] = Wr[S * p];
@@ -291,25 +326,39 @@ __global__ void __launch_bounds__(RowN<N, MODE>::BLOCK, RowN<N, MODE>::MINB) row
         ky[i] = (float)(iy[i] - K);
         ly[i] = ky[i] * ky[i] + sc[i].kz * sc[i].kz;
       }
-      // the new stage value replaces the first staged array, element by element
+      // the new stage value replaces the staged array, element by element; the others come from L2,
+      // a chunk of slots ahead of their use
+      constexpr int CH = 6;
+      cx<float> nx[2][CH][2];
+      auto fetch = [&](int q0, cx<float>(&d)[CH][2]) {
 #pragma unroll
-      for (int q = 0; q < SLOTS; ++q) {
-        const int e = lane + 32 * q;
-        if (valid(e)) {
-          const int i = row_of(e), j = e - i * P;
-          const float fkx = (float)(j - K), fky = at(ky, i);
-          const StageCoef<float> cf = at(sc, i);
-          const float kz = cf.kz;
-          const float k1 = (c == 0 ? fky : (c == 1 ? kz : fkx)) * inv_n2;
-          const float k2 = (c == 0 ? kz : (c == 1 ? fkx : fky)) * inv_n2;
-          const cx<float> f = mul_i(B2[e] * k1 - B1[e] * k2);
-          const float lam = (fkx * fkx + at(ly, i)) * cf.inv_rm;
-          const float g = implicit_gain(cf.dt * 0.5f * lam);
-          cx<float> r[3];
+        for (int k = 0; k < CH; ++k)
 #pragma unroll
-          for (int t = 0; t < NPRE; ++t) r[t] = t < npre ? Q[t * SLOTS * 32 + e] : mk(0.f, 0.f);
-          Q[e] = stage_update_1<MODE>(cf, sa, at(cb, i) + j, g, cf.dt * lam, r, f,
-                                      xout ? xout + full_at(i, j) : nullptr);
+          for (int t = 1; t < NPRE; ++t) {
+            const int e = lane + 32 * (q0 + k);
+            d[k][t - 1] = q0 + k < SLOTS && valid(e) && t < npre ? *addr(t, row_of(e), e - row_of(e) * P) : mk(0.f, 0.f);
+          }
+      };
+      fetch(0, nx[0]);
+#pragma unroll
+      for (int q0 = 0; q0 < SLOTS; q0 += CH) {
+        fetch(q0 + CH, nx[(q0 / CH + 1) & 1]);
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+          const int q = q0 + k, e = lane + 32 * q;
+          if (q < SLOTS && valid(e)) {
+            const int i = row_of(e), j = e - i * P;
+            const float fkx = (float)(j - K), fky = at(ky, i);
+            const StageCoef<float> cf = at(sc, i);
+            const float kz = cf.kz;
+            const float k1 = (c == 0 ? fky : (c == 1 ? kz : fkx)) * inv_n2;
+            const float k2 = (c == 0 ? kz : (c == 1 ? fkx : fky)) * inv_n2;
+            const cx<float> f = mul_i(B2[e] * k1 - B1[e] * k2);
+            const float lam = (fkx * fkx + at(ly, i)) * cf.inv_rm;
+            const float g = fused_gain(cf.dt * 0.5f * lam);
+            const cx<float> r[3] = {Q[e], nx[(q0 / CH) & 1][k][0], nx[(q0 / CH) & 1][k][1]};
+            Q[e] = rown_update<MODE>(cf, sa, at(cb, i) + j, g, cf.dt * lam, r, f, xout ? xout + full_at(i, j) : nullptr);
+          }
         }
       }
       __syncthreads();                                     // the curl is read before B is rewritten

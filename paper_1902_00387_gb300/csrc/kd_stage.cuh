@@ -92,6 +92,15 @@ __device__ __forceinline__ cx<double> implicit_solve(cx<double> t, double g) {
   return mk(__fma_rn(-t.x, g, t.x), __fma_rn(-t.y, g, t.y));
 }
 
+// h / (1 + h) for h >= 0 (implicit_gain): in complex64 an approximate reciprocal and one
+// residual correction of the quotient (Markstein's step), which rounds it as the division does but
+// for rare last-bit cases, without the division's range checks (1 + h is never tiny or huge).
+__device__ __forceinline__ float fused_gain(float h) {
+  const float d = 1.f + h, r = __fdividef(1.f, d), q = h * r;
+  return __fmaf_rn(__fmaf_rn(-q, d, h), r, q);
+}
+__device__ __forceinline__ double fused_gain(double h) { return implicit_gain(h); }
+
 // Stage arrays with no aliasing between them, so that loads of several points can be
 // issued before the stores of earlier points.
 //

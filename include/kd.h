@@ -238,8 +238,8 @@ kd_status kd_parareal_resume(kd_ctx* ctx, const double* u_init, int k_done, doub
                              double tol, double* u_slices, kd_parareal_stats* stats);
 
 /* Thread blocks per cluster of the persistent coarse solver (coarse sets up to 88 modes
- * a side): 0 = the default (a batch of fields that fits the GPU in clusters of 16: ~3 rows
- * per block, up to 16 blocks; larger batches: ~6 rows per block, at most 8), else 1..8 (1..16 where the
+ * a side): 0 = the default (by the batch: a few fields take up to 16 blocks each, many the
+ * size that needs the least waves of clusters), else 1..8 (1..16 where the
  * device allows non-portable cluster sizes) when the rows of a block fit its
  * modes-per-thread budget.  Fewer blocks mean cheaper cluster
  * barriers and more work per block.  KD_EINVAL if the coarse set does not fit. */

@@ -15,6 +15,8 @@
 // Layout: the stage values live in shared memory with a one-mode ring of zeros around
 // the kept square; the IMEX RK443 state X0 and accumulators R2..R4 of each mode live in
 // the registers of the thread that owns the mode.
+#include <mutex>
+
 #include "kd_coarse_kernel.cuh"
 
 namespace kd {
@@ -46,9 +48,7 @@ static size_t cluster_smem(int prec, int P, int nsteps, int* phase_slots, int re
   return base + (size_t)slots * es;
 }
 
-// modes per thread needed for a P-row square (0: unsupported)
-// modes per thread of a block (1: CCB1 threads; 2, 4: CCB threads); 0 if the rows of a
-// block do not fit
+// variant of the kernel that holds the rows of a block (cluster_kernel); 0 if none does
 static int modes_per_thread(int P, int req = 0) {
   int CS, H;
   cluster_shape(P, &CS, &H, req);
@@ -104,22 +104,67 @@ static int sm_count() {
   return sms;
 }
 
-// Default cluster size: the per-stage time is a fixed barrier / latency part plus a part
-// proportional to the rows of a block, so a few fields take the largest clusters that all
-// fit on the GPU at once (~3 rows per block, up to 16 blocks); larger batches keep ~6 rows
-// per block (at most 8) so that more clusters run concurrently.
-static int auto_cluster(int P, int batch) {
-  if (g_max_cluster >= 16 && batch * 16 <= sm_count()) {
-    const int cs = (P + 2) / 3 < 16 ? (P + 2) / 3 : 16;
-    if (cs > 8 && coarse_cluster_fits(P, cs)) return cs;
+// Clusters of a shape that run at once, asked of the runtime once per device, precision, square
+// and cluster size (with the whole phase table that a block may stage).
+template <typename T>
+static int active_clusters(int P, int cs) {
+  static std::mutex m;
+  static short cache[16][128][17];   // clusters + 1; 0: not asked yet
+  int dev = 0, n = 0, slots = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(m);
+  if (dev < 16 && cache[dev][P][cs]) return cache[dev][P][cs] - 1;
+  const int v = modes_per_thread(P, cs);
+  cudaLaunchAttribute at[1];
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)cs, 1, 1);
+  cfg.blockDim = dim3(cluster_threads<T>(v), 1, 1);
+  cfg.dynamicSmemBytes = cluster_smem(sizeof(T) == 4 ? 0 : 1, P, kMaxPhaseSlots / 16, &slots, cs);
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&n, cluster_kernel<T, 0>(v), &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
   }
-  return modes_per_thread(P) > 0 ? 0 : min_fitting_cluster(P);
+  if (dev < 16) cache[dev][P][cs] = (short)(n < 32000 ? n + 1 : 32000);
+  return n;
+}
+
+// Default cluster size of a batch: the least waves times a step's time, which is a fixed part
+// (barriers and latencies) plus one that grows with the modes an SM holds (FP32, one field, us:
+// 85 x 85 3.4 at 16 blocks, 4.4 at 11, 4.9 at 8; 43 x 43 2.6 at 11, 3.3 at 4, 4.9 at 2).  So a few
+// fields take the largest clusters; 64 of 85 x 85 take 10 blocks in 4 waves (22.4; 23.7 at 9, 24.7
+// at 8, 33.8 at 16), 64 of 43 x 43 two blocks and one wave (5.0; 12.9 at 8, the former rule's), 16
+// of 65 x 65 six (4.5; 8.3 at 8).  FP64 arithmetic bounds FP64 steps (85 x 85: 64 at 16 blocks, 118
+// at 8; 16 fields 177 at 11 blocks, 237 at 8).
+template <typename T>
+static int auto_cluster(int P, int batch) {
+  int best = 0;
+  double best_t = 0.0;
+  for (int cs = 1; cs <= g_max_cluster && cs <= P; ++cs) {
+    int CS, H;
+    cluster_shape(P, &CS, &H, cs);
+    if (!coarse_cluster_fits(P, cs) || (P + H - 1) / H != cs) continue;   // no block without rows
+    const int cap = active_clusters<T>(P, cs);
+    if (cap <= 0) continue;
+    const int at_once = batch < cap ? batch : cap, co = (at_once * cs + sm_count() - 1) / sm_count();
+    const double t = (double)((batch + cap - 1) / cap) * (2.2 + (sizeof(T) == 4 ? 0.0025 : 0.126) * co * H * P);
+    if (!best || t < best_t) {
+      best = cs;
+      best_t = t;
+    }
+  }
+  return best ? best : modes_per_thread(P) > 0 ? 0 : min_fitting_cluster(P);
 }
 
 template <typename T>
 static int launch_cluster(const CoarseArgs& a0, int batch, cudaStream_t st) {
   CoarseArgs a = a0;
-  const int req = a.cluster > 0 && coarse_cluster_fits(a.Pc, a.cluster) ? a.cluster : auto_cluster(a.Pc, batch);
+  const int req = a.cluster > 0 && coarse_cluster_fits(a.Pc, a.cluster) ? a.cluster : auto_cluster<T>(a.Pc, batch);
   int CS, H, slots;
   cluster_shape(a.Pc, &CS, &H, req);
   const size_t sm = cluster_smem(sizeof(T) == 4 ? 0 : 1, a.Pc, a.nsteps, &slots, req);
@@ -127,7 +172,7 @@ static int launch_cluster(const CoarseArgs& a0, int batch, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(CS * batch), 1, 1);
   const int mpt = modes_per_thread(a.Pc, req);
-  cfg.blockDim = dim3(mpt == 1 ? CCB1 : CCB, 1, 1);
+  cfg.blockDim = dim3(cluster_threads<T>(mpt), 1, 1);
   cfg.dynamicSmemBytes = sm;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];

@@ -46,8 +46,7 @@ __device__ __forceinline__ UHat<T> uhat(T A, const Phase<T>& p) {
 // below, double-buffered: a stage reads buffer `cur`, writes its new rows into `nxt`
 // locally and its first / last row into the neighbours' halo rows of `nxt` through
 // distributed shared memory, then one cluster barrier makes `nxt` current.
-constexpr int CCB = 256;   // threads per block of the cluster kernel (MPT = 2, 4)
-constexpr int CCB1 = 512;  // threads per block with one mode per thread
+constexpr int CCB = 256, CCB1 = 512;   // threads per block of the cluster kernel's variants
 
 // Halo exchange after each stage (CoarseArgs::halo).  0 (default): the first and last rows
 // are stored into the neighbours' halo rows through distributed shared memory, then one
@@ -114,9 +113,6 @@ __global__ void __launch_bounds__(NT) coarse_cluster_kernel(CoarseArgs a, int CS
   const long slot = a.map ? (long)a.map[b] : (long)b;
   const double* Un = a.Un + slot * lenf2;
   const double* Uprev = a.Uprev ? a.Uprev + (a.map ? slot * lenf2 : 0) : nullptr;
-  const double* Fv = a.Fv ? a.Fv + (a.map ? slot * lenf2 : 0) : nullptr;
-  double* Unext = a.Unext ? a.Unext + (a.map ? (slot + 1) * lenf2 : 0) : nullptr;
-  double* sig = a.sigma_out ? a.sigma_out + (a.map ? 3L * b : 0) : nullptr;
   const int nsteps = a.steps ? a.steps[b] : a.nsteps;
   for (int i = threadIdx.x; i < 2 * bufsz; i += NT) buf[i] = mk(T(0), T(0));
   const bool stage_ph = a.phases && a.nsteps * 16 <= a.phase_smem;
@@ -343,7 +339,7 @@ __global__ void __launch_bounds__(NT) coarse_cluster_kernel(CoarseArgs a, int CS
             }
           }
           // no pushes after the last stage, nor once a halo wait of this block timed out
-          const bool send = !pull && g + 1 < G && !*(volatile int*)&s_bad;
+          const bool send = !pull && g + 1 < G && !(p2p && *(volatile int*)&s_bad);
 #pragma unroll
           for (int c = 0; c < 3; ++c) put(cur ^ 1, (g + 1) & 3, send, i, c, xn[c]);
         }
@@ -378,6 +374,9 @@ __global__ void __launch_bounds__(NT) coarse_cluster_kernel(CoarseArgs a, int CS
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // the final stage everywhere
   }
 
+  const double* Fv = a.Fv ? a.Fv + (a.map ? slot * lenf2 : 0) : nullptr;
+  double* Unext = a.Unext ? a.Unext + (a.map ? (slot + 1) * lenf2 : 0) : nullptr;
+  double* sig = a.sigma_out ? a.sigma_out + (a.map ? 3L * b : 0) : nullptr;
   // outputs from the final stage value (buffer `cur`), by stripe
   const cx<T>* Xf = buf + cur * bufsz;
   if (a.mode == COARSE_OUT) {
@@ -475,34 +474,50 @@ __global__ void __launch_bounds__(NT) coarse_cluster_kernel(CoarseArgs a, int CS
 }
 
 
-// the three modes-per-thread variants of one halo exchange
+
+// The variants of one halo exchange by the modes a block holds: up to 512 one a thread, up to 256
+// two (two blocks share an SM), up to 1024 two in FP32 and four in FP64, whose registers hold two.
+// In FP32 16 warps with two modes hide their latencies better than 8 with four: 64 fields of
+// 85 x 85, 11 rows a block, 27.7 us a step with four modes a thread.
+template <typename T>
+constexpr int kBigM = sizeof(T) == 4 ? 2 : 4;
+template <typename T>
+constexpr int kBigT = sizeof(T) == 4 ? CCB1 : CCB;
+
+// variant v (modes_per_thread): 1, 2, 4 as the modes a thread of it would hold at 512, 256, 256
+template <typename T, int HALO>
+const void* cluster_kernel(int v) {
+  return v == 1   ? (const void*)coarse_cluster_kernel<T, 1, CCB1, HALO>
+         : v == 2 ? (const void*)coarse_cluster_kernel<T, 2, CCB, HALO>
+                  : (const void*)coarse_cluster_kernel<T, kBigM<T>, kBigT<T>, HALO>;
+}
+
+template <typename T>
+int cluster_threads(int v) {
+  return v == 1 ? CCB1 : v == 2 ? CCB : kBigT<T>;
+}
+
 template <typename T, int HALO>
 cudaError_t cluster_allow_nonportable() {
-  cudaError_t e = cudaFuncSetAttribute(coarse_cluster_kernel<T, 1, CCB1, HALO>,
-                                       cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(coarse_cluster_kernel<T, 2, CCB, HALO>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(coarse_cluster_kernel<T, 4, CCB, HALO>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaError_t e = cudaSuccess;
+  for (int v = 1; v <= 4 && e == cudaSuccess; v *= 2)
+    e = cudaFuncSetAttribute(cluster_kernel<T, HALO>(v), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   return e;
 }
 
 template <typename T, int HALO>
 cudaError_t cluster_set_smem(int bytes) {
-  cudaError_t e =
-      cudaFuncSetAttribute(coarse_cluster_kernel<T, 1, CCB1, HALO>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(coarse_cluster_kernel<T, 2, CCB, HALO>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(coarse_cluster_kernel<T, 4, CCB, HALO>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = cudaSuccess;
+  for (int v = 1; v <= 4 && e == cudaSuccess; v *= 2)
+    e = cudaFuncSetAttribute(cluster_kernel<T, HALO>(v), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   return e;
 }
 
 template <typename T, int HALO>
-cudaError_t cluster_launch(const cudaLaunchConfig_t& cfg, int mpt, const CoarseArgs& a, int CS, int H) {
-  return mpt == 1   ? cudaLaunchKernelEx(&cfg, coarse_cluster_kernel<T, 1, CCB1, HALO>, a, CS, H)
-         : mpt == 2 ? cudaLaunchKernelEx(&cfg, coarse_cluster_kernel<T, 2, CCB, HALO>, a, CS, H)
-                    : cudaLaunchKernelEx(&cfg, coarse_cluster_kernel<T, 4, CCB, HALO>, a, CS, H);
+cudaError_t cluster_launch(const cudaLaunchConfig_t& cfg, int v, const CoarseArgs& a, int CS, int H) {
+  return v == 1   ? cudaLaunchKernelEx(&cfg, coarse_cluster_kernel<T, 1, CCB1, HALO>, a, CS, H)
+         : v == 2 ? cudaLaunchKernelEx(&cfg, coarse_cluster_kernel<T, 2, CCB, HALO>, a, CS, H)
+                  : cudaLaunchKernelEx(&cfg, coarse_cluster_kernel<T, kBigM<T>, kBigT<T>, HALO>, a, CS, H);
 }
 
 }  // namespace kd

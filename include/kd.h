@@ -476,7 +476,9 @@ kd_status kd_selftest_wait(int arrive, double max_ms, void* cuda_stream);
  * the paper.  The limit caps the device bytes the context holds in its own buffers (grid
  * tables, fine and coarse workspaces, Parareal arrays, staging; not CUDA's own objects
  * such as streams, events and graph executables, nor the static array of
- * kd_fine_batched_static).  max_bytes = 0 removes it (the default); a limit below what the
+ * kd_fine_batched_static).  Training buffers that the context keeps for its next training
+ * call (at most 1 GiB) count as held and are released before a request is refused or, on a
+ * GPU that is out of memory, fails.  max_bytes = 0 removes it (the default); a limit below what the
  * context already holds keeps those buffers and refuses new ones.  A call that needs a
  * buffer beyond the limit returns KD_ENOMEM, as a failed cudaMalloc does, with
  * kd_last_error naming the buffer, its size, the bytes held and the limit; the context

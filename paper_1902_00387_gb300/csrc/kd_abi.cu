@@ -45,15 +45,42 @@ bool valid_n(int n) {
   return n == 16 || n == 32 || n == 64 || n == 128 || n == 256 || n == 512 || n == 1024;
 }
 
+// Buffers that dkeep left are given to requests of their size, and given back to CUDA before
+// any request fails.
+static void drop_spares(kd_ctx* ctx, size_t keep) {
+  while (ctx->spare_bytes > keep) {
+    const size_t i = ctx->spare.front();
+    ctx->spare.erase(ctx->spare.begin());
+    ctx->spare_bytes -= ctx->alloc_sizes[i];
+    dfree(ctx, ctx->allocs[i]);
+  }
+}
+
 kd_status dalloc(kd_ctx* ctx, void** p, size_t bytes, const char* what) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
+  if (ctx->alloc_limit && ctx->alloc_held > ctx->alloc_limit) drop_spares(ctx, 0);   // no use of them beyond the limit
+  for (size_t k = 0; k < ctx->spare.size(); ++k)
+    if (ctx->alloc_sizes[ctx->spare[k]] == bytes) {
+      *p = ctx->allocs[ctx->spare[k]];
+      ctx->spare.erase(ctx->spare.begin() + k);
+      ctx->spare_bytes -= bytes;
+      ++ctx->alloc_gen;
+      return KD_OK;
+    }
+  if (ctx->alloc_limit && (bytes > ctx->alloc_limit || ctx->alloc_held > ctx->alloc_limit - bytes))
+    drop_spares(ctx, 0);
   // the context's allocation limit refuses the buffer as a failed cudaMalloc would
   if (ctx->alloc_limit && (bytes > ctx->alloc_limit || ctx->alloc_held > ctx->alloc_limit - bytes))
     return fail(ctx, KD_ENOMEM, std::string("allocation limit: ") + what + " (" + std::to_string(bytes) +
                                     " B) with " + std::to_string(ctx->alloc_held) + " B held exceeds the limit of " +
                                     std::to_string(ctx->alloc_limit) + " B");
   cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess && ctx->spare_bytes) {
+    cudaGetLastError();
+    drop_spares(ctx, 0);
+    e = cudaMalloc(p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(ctx, KD_ENOMEM, std::string("cudaMalloc ") + what + " (" + std::to_string(bytes) + " B): " +
@@ -84,6 +111,21 @@ void dfree(kd_ctx* ctx, void* p) {
       ctx->alloc_sizes[i] = 0;
       return;
     }
+}
+
+// Release a buffer of a synchronous call whose work on it has finished, keeping it for the next
+// call: cudaMalloc and cudaFree of the training buffers (0.7 GB at 49 modes) take longer than
+// the GEMMs on them.  At most 1 GiB is kept, the newest; the context gives it back when an
+// allocation would fail and at its end.
+void dkeep(kd_ctx* ctx, void* p) {
+  constexpr size_t LIMIT = (size_t)1 << 30;
+  for (size_t i = 0; p && i < ctx->allocs.size(); ++i)
+    if (ctx->allocs[i] == p) {
+      ctx->spare.push_back(i);
+      ctx->spare_bytes += ctx->alloc_sizes[i];
+      break;
+    }
+  drop_spares(ctx, LIMIT);
 }
 
 kd_status make_tables(kd_ctx* ctx, Tables& t, int n, int prec) {
@@ -1111,15 +1153,15 @@ kd_status kd_coarse(kd_ctx* ctx, const double* b_in, double* b_out, const double
   if (batch < 0 || nsteps < 0) return fail(ctx, KD_EINVAL, "kd_coarse: negative batch or nsteps");
   if (batch == 0) return KD_OK;
   const int n = ctx->p.n, nc = ctx->p.n_coarse, pc = ctx->p.prec_coarse;
-  kd_status s = ensure_ws(ctx, ctx->ws_c, nc, pc, batch);
-  if (s != KD_OK) return s;
+  kd_status s;
   // full (n) -> coarse compact via the staging buffer holding the fine compact form
   const size_t fcb = (size_t)batch * compact_len(n) * 16;
   if ((s = ensure_full_tmp(ctx, fcb)) != KD_OK) return s;
   KD_LAUNCH(full_to_compact(KD_C128, b_in, KD_C128, ctx->full_tmp, batch, n, ctx->st), "pack");
   if (coarse_conv_supported(ctx->cP) && nsteps > 0) {
-    // persistent convolution-form solve, one block per field; result in ws_c.X as FP64
-    if ((s = ensure_ws(ctx, ctx->ws_c, nc, KD_C128, batch)) != KD_OK) return s;
+    // persistent convolution-form solve, one cluster per field; result in FP64 staging of its own:
+    // a workspace shared with the other precision would be allocated anew by each call
+    if ((s = ensure_conv_tmp(ctx, (size_t)batch * compact_len(nc) * 16)) != KD_OK) return s;
     FineArgs pa = fine_args(ctx, ctx->ws_c, ctx->tab_c, nc, batch, ctx->p.dt_coarse, t0);
     const size_t need = phase_table_bytes(pc, batch, nsteps);
     if (ctx->p.flow == KD_FLOW_GALLOWAY_PROCTOR && ctx->ph_c_bytes < need) {
@@ -1135,12 +1177,13 @@ kd_status kd_coarse(kd_ctx* ctx, const double* b_in, double* b_out, const double
     c.phases = ctx->p.flow == KD_FLOW_GALLOWAY_PROCTOR ? ctx->ph_c : nullptr;
     c.Un = (const double*)ctx->full_tmp;
     c.mode = COARSE_OUT;
-    c.g64 = (double*)ctx->ws_c.X;
+    c.g64 = (double*)ctx->conv_tmp;
     KD_LAUNCH(coarse_conv_launch(pc, c, batch, ctx->st), "coarse solve");
-    KD_LAUNCH(compact_resample(KD_C128, ctx->ws_c.X, nc, KD_C128, ctx->full_tmp, n, batch, ctx->st), "prolong");
+    KD_LAUNCH(compact_resample(KD_C128, ctx->conv_tmp, nc, KD_C128, ctx->full_tmp, n, batch, ctx->st), "prolong");
     KD_LAUNCH(compact_to_full(KD_C128, ctx->full_tmp, KD_C128, b_out, batch, n, ctx->st), "unpack");
     return KD_OK;
   }
+  if ((s = ensure_ws(ctx, ctx->ws_c, nc, pc, batch)) != KD_OK) return s;
   KD_LAUNCH(compact_resample(KD_C128, ctx->full_tmp, n, pc, ctx->ws_c.X, nc, batch, ctx->st), "restrict");
   FineArgs a = fine_args(ctx, ctx->ws_c, ctx->tab_c, nc, batch, ctx->p.dt_coarse, t0);
   if ((s = with_phases(ctx, ctx->ws_c, a, nsteps)) != KD_OK) return s;
@@ -1551,7 +1594,7 @@ kd_status check_gemm(kd_ctx* ctx, const TrainBufs& b) {
 
 void free_train_bufs(kd_ctx* ctx, TrainBufs& b) {
   void* all[] = {b.xp, b.yp, b.yT, b.C1, b.C2, b.Xs, b.XtT, b.A2, b.Wbf, b.err};
-  for (void* p : all) dfree(ctx, p);
+  for (void* p : all) dkeep(ctx, p);
   b = TrainBufs();
 }
 
@@ -1561,13 +1604,18 @@ kd_status load_pairs(kd_ctx* ctx, TrainBufs& b, const float* x, const float* y, 
   const size_t vb = 2 * (size_t)nc * 4;
   KD_CUDA(cudaMemsetAsync(b.xp, 0, mp * vb, ctx->st), "memset");
   KD_CUDA(cudaMemsetAsync(b.yp, 0, mp * vb, ctx->st), "memset");
-  for (size_t t = 0; t < idx.size(); ++t) {
-    KD_CUDA(cudaMemcpyAsync((char*)b.xp + t * vb, (const char*)x + (size_t)idx[t] * vb, vb, cudaMemcpyDeviceToDevice,
-                            ctx->st),
-            "gather x");
-    KD_CUDA(cudaMemcpyAsync((char*)b.yp + t * vb, (const char*)y + (size_t)idx[t] * vb, vb, cudaMemcpyDeviceToDevice,
-                            ctx->st),
-            "gather y");
+  for (size_t t = 0; t < idx.size();) {
+    // the pairs of a phase are consecutive or, when the phases take turns, evenly spaced: one copy
+    // for as many as have the same spacing
+    size_t e = t + 1;
+    size_t gap = e < idx.size() && idx[e] > idx[t] ? idx[e] - idx[t] : 1;
+    if (gap * vb > ((size_t)1 << 30)) gap = 1;                 // a copy's pitch is below 2 GB
+    while (e < idx.size() && idx[e] == idx[e - 1] + (int)gap) ++e;
+    for (int v = 0; v < 2; ++v)
+      KD_CUDA(cudaMemcpy2DAsync((char*)(v ? b.yp : b.xp) + t * vb, vb, (const char*)(v ? y : x) + (size_t)idx[t] * vb,
+                                gap * vb, vb, e - t, cudaMemcpyDeviceToDevice, ctx->st),
+              v ? "gather y" : "gather x");
+    t = e;
   }
   KD_LAUNCH(learned_pack_x(b.xp, mp, mp, nc, (nc + 7) & ~7, b.Xs, b.XtT, ctx->st), "pack x");
   KD_LAUNCH(learned_transpose_y(b.yp, mp, mp, nc, b.yT, ctx->st), "transpose y");

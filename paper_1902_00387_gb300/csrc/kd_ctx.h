@@ -106,6 +106,8 @@ struct kd_ctx {
   std::vector<size_t> alloc_sizes;
   size_t alloc_held = 0;
   size_t alloc_limit = 0;
+  std::vector<size_t> spare;  // entries of allocs that dkeep released, oldest first
+  size_t spare_bytes = 0;
   std::string err;
   long long launches = 0;     // kernels launched by this context
   int cK = 0, cP = 0;         // coarse mode set k in [-cK, cP - cK)^2
@@ -167,6 +169,7 @@ inline long compact_len(int n) { return 3L * kept(n) * kept(n); }  // complex en
 int steps_for(double dT, double dt);
 kd_status dalloc(kd_ctx* ctx, void** p, size_t bytes, const char* what);
 void dfree(kd_ctx* ctx, void* p);
+void dkeep(kd_ctx* ctx, void* p);
 kd_status make_tables(kd_ctx* ctx, Tables& t, int n, int prec);
 kd_status ensure_ws(kd_ctx* ctx, FineWs& w, int n, int prec, long batch);
 kd::FineArgs fine_args(const kd_ctx* ctx, const FineWs& w, const Tables& t, int n, long batch, double dt,

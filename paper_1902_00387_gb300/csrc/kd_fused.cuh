@@ -20,9 +20,12 @@
 // the launches, by few warps in flight and by L2 round trips of the mixed field.  Bound now: the
 // instruction issue of the passes (90% in the column pass, 870 instructions a 96-point column)
 // for a batch, the chain of a stage (~11 k cycles at 128^2, two cluster barriers among them) for
-// a few fields.  Measured, us a step, against the two-kernel plans: 128^2 complex64, 64 fields 76
-// (137), one 24 (39); 64^2 x 64 22 (81); 32^2 x 8 13 (62); 160^2 x 10 on 128 points 44 (82); 192^2
-// x 100 464 (889); 256^2 x 128 745 (931); complex128 32^2 x 8 57 (314), 128^2 x 64 1970 (2508).
+// a few fields.  Measured, us a step, against the two-kernel plans: 128^2 complex64, 64 fields 72
+// (137), one 23 (39); 64^2 x 64 22 (81); 32^2 x 8 14 (62); 160^2 x 10 on 128 points 43 (82); 192^2
+// x 100 425 (889); 256^2 x 128 745 (931); complex128 32^2 x 8 57 (314), 128^2 x 64 1970 (2508).
+// In complex64 stage 0 stores its explicit term alone, and stage 1 forms the accumulators from it
+// and the state: 14 compact arrays a step instead of 17 (128^2 x 64 72.1 us instead of 75.6, 256^2 x
+// 128 745 instead of 777).  Complex128 is bound by FP64 arithmetic and keeps the accumulators.
 // Tried and slower: 12 or 24 values a lane with one transpose through shared memory, which
 // executes fewer instructions but fits fewer and longer chains of warps (80 and 100 us at 128^2
 // x 64); x in q + R rev(l), whose accesses to other blocks split into three times the sectors.
@@ -241,16 +244,32 @@ __device__ __forceinline__ cx<T>& fused_at(cx<T>* p, unsigned o) {
 
 // One component of one IMEX RK443 stage (the expressions of stage_update, kd_stage.cuh): f =
 // F_c(X_j); r the arrays read: X (stage 0), R2 R3 R4 (1), R3 R4 (2), R4 X Xlo (3); o: where the
-// arrays written go: R2 R3 R4; R3 R4; R4; X Xlo; stored where `on`.  Returns X_{j+1}.
+// arrays written go: R2 R3 R4; R3 R4; R4; X Xlo; stored where `on`.  In complex64 stage 0 writes
+// f to R2 only and stage 1 reads X and f.  Returns X_{j+1}.
 template <int MODE, typename T>
 __device__ __forceinline__ cx<T> fused_update(cx<T>* o0, cx<T>* o1, cx<T>* o2, bool on, T dt, T g, T dl, cx<T> f,
                                               const cx<T>* r) {
   if constexpr (MODE == 0) {
     const cx<T> t = wt_fma(f, dt * T(0.5), r[0]), x = wt_fma(t, -g, t);
+    if constexpr (sizeof(T) == 4) {
+      if (on) *o0 = f;
+      return x;
+    }
     if (on) {
       *o0 = wt_fma(x, dl * T(-1.0 / 6.0), wt_fma(f, dt * T(11.0 / 18.0), r[0]));
       *o1 = wt_fma(x, dl * T(0.5), wt_fma(f, dt * T(5.0 / 6.0), r[0]));
       *o2 = wt_fma(x, dl * T(-1.5), f * (dt * T(0.25)));
+    }
+    return x;
+  } else if constexpr (MODE == 1 && sizeof(T) == 4) {   // r: X, the explicit term of stage 0
+    const cx<T> t0 = wt_fma(r[1], dt * T(0.5), r[0]), x1 = wt_fma(t0, -g, t0);
+    const cx<T> a[3] = {wt_fma(x1, dl * T(-1.0 / 6.0), wt_fma(r[1], dt * T(11.0 / 18.0), r[0])),
+                        wt_fma(x1, dl * T(0.5), wt_fma(r[1], dt * T(5.0 / 6.0), r[0])),
+                        wt_fma(x1, dl * T(-1.5), r[1] * (dt * T(0.25)))};
+    const cx<T> t = wt_fma(f, dt * T(1.0 / 18.0), a[0]), x = wt_fma(t, -g, t);
+    if (on) {
+      *o0 = wt_fma(x, dl * T(-0.5), wt_fma(f, dt * T(-5.0 / 6.0), a[1]));
+      *o1 = wt_fma(x, dl * T(1.5), wt_fma(f, dt * T(1.75), a[2]));
     }
     return x;
   } else if constexpr (MODE == 1) {
@@ -355,9 +374,10 @@ __global__ void __launch_bounds__(32 * FusedStep<T, L, R>::MAXW, 1) fused_kernel
   // stage arrays are loaded before the transform, which covers their latency (L2), those of AHEAD
   // registers at a time.
   auto row_pass = [&](int stage, bool more, bool lo_valid) {
-    const cx<T>* p0 = stage == 0 ? Xp : (stage == 1 ? R2 : (stage == 2 ? R3 : R4));
-    const cx<T>* p1 = stage == 1 ? R3 : (stage == 2 ? R4 : (stage == 3 ? Xp : nullptr));
-    const cx<T>* p2 = stage == 1 ? R4 : (stage == 3 && lo_valid ? Xl : nullptr);
+    constexpr bool f0 = sizeof(T) == 4;            // stage 0 leaves its explicit term in R2
+    const cx<T>* p0 = stage == 0 || (stage == 1 && f0) ? Xp : (stage == 1 ? R2 : (stage == 2 ? R3 : R4));
+    const cx<T>* p1 = stage == 1 ? (f0 ? R2 : R3) : (stage == 2 ? R4 : (stage == 3 ? Xp : nullptr));
+    const cx<T>* p2 = stage == 1 && !f0 ? R4 : (stage == 3 && lo_valid ? Xl : nullptr);
     for (int t = warp; t * TPW < rows; t += nw) {
       const bool ok = t * TPW + grp < rows;
       const int iy = y0 + min(t * TPW + grp, rows - 1);

@@ -281,14 +281,27 @@ class ClockSampler:
 # ---------------------------------------------------------------- roofline
 def col_row_bytes(n, batch_slices):
     """Algorithmic bytes of one column launch and of one row launch (complex64):
-    the column pass reads and writes the mixed field (3 x P x n); the row pass reads
-    and writes it too and touches 3.5 compact spectral arrays (3 x P x P) on average
-    over the four stages (stage reads + writes: 4, 5, 3, 2)."""
+    the column pass reads and writes the mixed field (3 x P x N); the row pass reads
+    and writes it too and touches compact spectral arrays (3 x P x P) over the four
+    stages.  Sides 512 and 1024 work on N = 3n/4 points and move 2, 4, 3, 3 compact
+    arrays at the stages (the state; its low part is not counted), the two-kernel step
+    of the other sides on N = n with 4, 5, 3, 2."""
     K = n // 3
     P = 2 * K + 1
-    mixed = 3 * P * n * 8
+    narrow = n in (512, 1024)
+    mixed = 3 * P * (3 * n // 4 if narrow else n) * 8
     spec = 3 * P * P * 8
-    return 2 * mixed * batch_slices, (2 * mixed + 3.5 * spec) * batch_slices
+    return 2 * mixed * batch_slices, (2 * mixed + (3.0 if narrow else 3.5) * spec) * batch_slices
+
+
+FUSED_PASSES = 14   # compact arrays read or written by a step, the low part of the state counted
+
+
+def fused_bytes(n, batch_slices):
+    """Algorithmic bytes of one step of the persistent fused kernel (complex64): the
+    compact arrays of the four stages; the mixed field stays in shared memory."""
+    P = 2 * (n // 3) + 1
+    return FUSED_PASSES * 3 * P * P * 8 * batch_slices
 
 
 # --------------------------------------------------- learned coarse propagator run
@@ -1078,15 +1091,17 @@ def parareal_c2(args, env, embedded):
     S = st.n_fine_steps
     # fine-sweep batches over one solve: slices k-1..N-1 in iteration k
     batches = [N - min(k - 1, N - 1) for k in range(1, st.k_con + 1)]
+    fused = prof_n[0] == 0 and prof_n[1] > 0     # the persistent step: one launch a sweep, all its steps
     col_b = sum(col_row_bytes(n, b)[0] * 4 * S for b in batches) * prof_steps
-    row_b = sum(col_row_bytes(n, b)[1] * 4 * S for b in batches) * prof_steps
+    row_b = sum((fused_bytes(n, b) if fused else col_row_bytes(n, b)[1] * 4) * S for b in batches) * prof_steps
     kid = 0 if prof_ms[0] >= prof_ms[1] else 1
+    kname = "persistent fused step" if fused else ("fine column kernel", "fine row kernel")[kid]
     kbytes = (col_b, row_b)[kid]
     achieved = kbytes / (prof_ms[kid] / 1e3) / 1e9 if prof_ms[kid] > 0 else 0.0
     fine_units = 3 * n * n * S * sum(batches) * steps
     fine_rate = fine_units / (sum(x.ms_fine for x in stats) / 1e3) / 1e6
     if args.fine_operator == "fft":
-        roof = {"bound": "latency (L2-resident)", "kernel": ("fine column kernel", "fine row kernel")[kid],
+        roof = {"bound": "issue and latency (L2-resident)", "kernel": kname,
                 "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
                 "traffic": None, "algorithmic_bytes_per_launch": kbytes / max(1, prof_n[kid]), "peak_kind": peak_kind,
                 "avg_launch_us": 1e3 * prof_ms[kid] / max(1, prof_n[kid]), "launches": prof_n[kid],
@@ -1142,15 +1157,15 @@ def run_parareal(args):
 
 # ------------------------------------------------- the default line: the fine step, c5
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the fine
-# kernels, from one ncu capture of the warp-transform plan (6, 7) at 1024^2 x 16 slices
+# kernels, from one ncu capture of the 768-point plan (6, 7) at 1024^2 x 16 slices
 # (one fine step: the 4 stage launches of each kernel), averaged over the stages and
 # scaled by 16 to a 256-slice launch (the traffic grows with the slices); keyed by the
 # kernel's name as the bench reports it and its variant (column variant for the column
 # kernel, row variant for the row kernel).  A variant without a capture of its current
 # code reports null.
 FINE_TRAFFIC = {
-    ("fine row kernel", 7): 16 * (1196.97 + 1374.91 + 1021.99 + 785.88) / 4 * 1e6,
-    ("fine column kernel", 6): 16 * (484.81 + 484.54 + 484.87 + 484.66) / 4 * 1e6,
+    ("fine row kernel", 7): 16 * (708.23 + 1067.68 + 888.26 + 867.54) / 4 * 1e6,
+    ("fine column kernel", 6): 16 * (362.56 + 362.71 + 362.48 + 362.83) / 4 * 1e6,
 }
 
 

@@ -29,7 +29,7 @@ constexpr int fit_blocks(int block, size_t smem, int min_regs) {
   return m < 1 ? 1 : m;
 }
 
-// Candidate tile shapes of the n <= 256 kernels (index 0 is the default plan).
+// Candidate tile shapes of the n <= 256 kernels (index 0: the plan of the calls that the fused step does not cover).
 template <typename T, int N>
 struct Shapes2 {
   static constexpr int R2 = Split<N>::R2;

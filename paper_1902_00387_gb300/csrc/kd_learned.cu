@@ -537,7 +537,8 @@ int learned_momentum(float* W, const float* W0, const float* C2, float* v, __nv_
 // stride ldc) and, in the same pass, per-block sums of |W - W0|^2 (partials[2 b], [2 b + 1] = 0).
 // Bound by HBM: four matrices cross it once (1.66 GB at nc = 7203).  With the gradient, its
 // unpacking and the norm in passes of their own over padded copies of W and W0, and those copies
-// allocated and filled by each call, a call with 256 pairs took 8.0 ms; it takes 2.1.  The norm is
+// allocated and filled by each call, a call with 256 pairs took 8.0 ms; with this pass 2.1 (1.07 with
+// the operands' buffers kept between calls).  The norm is
 // summed as an unevaluated pair of floats a thread (differences, squares and sums with their
 // rounding errors, ~45 bits) and in FP64 across threads: an FP64 product and sum per element
 // would be bound by the few FP64 units.

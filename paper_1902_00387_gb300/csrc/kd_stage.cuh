@@ -93,9 +93,11 @@ __device__ __forceinline__ cx<double> implicit_solve(cx<double> t, double g) {
 }
 
 // h / (1 + h) for h >= 0 (implicit_gain): in complex64 an approximate reciprocal and one
-// residual correction of the quotient (Markstein's step), which rounds it as the division does but
-// for rare last-bit cases, without the division's range checks (1 + h is never tiny or huge).
+// residual correction of the quotient (Markstein's step), without the division's range checks.
+// The value is the division's for every finite h (compared one by one by the tests).  h is held to
+// 2^60, whose factor is 1 like that of any h from 2^25 on: beyond 2^126 the approximate reciprocal is 0.
 __device__ __forceinline__ float fused_gain(float h) {
+  h = fminf(h, 0x1p60f);
   const float d = 1.f + h, r = __fdividef(1.f, d), q = h * r;
   return __fmaf_rn(__fmaf_rn(-q, d, h), r, q);
 }

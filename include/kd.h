@@ -529,14 +529,24 @@ kd_status kd_block_get_state(kd_ctx* ctx, int local_index, double* u);
  *
  * The fine step's column and row kernels exist in several variants per grid and
  * precision (columns or rows per thread block; the row kernel's stage update run from
- * shared memory or from registers).  A plan is the pair (col, row) of variant indices;
- * {0, 0} is the default, except on the complex64 grid n = 1024, whose default is the
- * warp-transform pair {5, 7}.  grid: 0 = the fine grid n, 1 = the coarse grid n_coarse. */
+ * shared memory or from registers).  A plan is the pair (col, row) of variant indices.
+ * Defaults in complex64: the persistent step at n = 16 (col 3), 32, 64, 128 (col 4) and
+ * 256 (col 6), to which row says nothing, and the pairs that step on 3n/4 points at
+ * n = 512 {5, 9} and n = 1024 {6, 7} (RK443; one of their indices beside another, or
+ * another scheme, means kernels on n points).  {0, 0} on every other grid.
+ *
+ * While no plan has been set or tuned, calls of a few fields in all take another default
+ * at n = 256 (up to 6 fields: {0, 9}) and n = 512 (up to 3: {6, 9}), whose kernels spread
+ * a field over the whole GPU.  Under one plan a field's values are the same bits in every
+ * batch; between two plans they differ by FP32 round-off.  A plan that was set or tuned is
+ * the one that runs in every call, so setting the default keeps the bits of small batches.
+ * grid: 0 = the fine grid n, 1 = the coarse grid n_coarse. */
 enum { KD_GRID_FINE = 0, KD_GRID_COARSE = 1 };
 
 /* Number of column / row variants of the context's grid.  KD_EINVAL for a bad grid. */
 kd_status kd_plan_variants(kd_ctx* ctx, int grid, int* n_col, int* n_row);
-/* Set / read the plan of a grid.  KD_EINVAL if an index is out of range. */
+/* Set / read the plan of a grid (kd_get_plan: the one of many fields while none was set).
+ * KD_EINVAL if an index is out of range. */
 kd_status kd_set_plan(kd_ctx* ctx, int grid, int col, int row);
 kd_status kd_get_plan(kd_ctx* ctx, int grid, int* col, int* row);
 

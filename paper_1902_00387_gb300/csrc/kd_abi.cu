@@ -311,9 +311,7 @@ int run_fine(kd_ctx* ctx, int g, int prec, const FineArgs& a, int nsteps, bool p
 
 FinePlan call_plan(const kd_ctx* ctx, long batch) {
   const int n = ctx->p.n, prec = ctx->p.prec_fine;
-  const FinePlan d = fine_default_plan(n, prec);
-  const bool is_default = ctx->plan[0].col == d.col && ctx->plan[0].row == d.row;
-  return is_default && batch <= fine_few(n, prec) ? fine_default_plan(n, prec, true) : ctx->plan[0];
+  return !ctx->plan_chosen && batch <= fine_few(n, prec) ? fine_default_plan(n, prec, true) : ctx->plan[0];
 }
 
 kd_status ensure_full_tmp(kd_ctx* ctx, size_t bytes) {
@@ -1414,13 +1412,13 @@ kd_status kd_fine_serial(kd_ctx* ctx, const double* b0, double T, int N, double*
   // one field at a time is a different launch shape from the batched sweeps: tune it once
   if (!conv_op(ctx) && !ctx->plan_serial_ok) {
     const FinePlan saved = ctx->plan[0];
+    const bool chosen = ctx->plan_chosen;
     if ((s = kd_autotune(ctx, KD_GRID_FINE, 1, 2, nullptr, nullptr)) != KD_OK) return s;
     ctx->plan_serial = ctx->plan[0];
     ctx->plan[0] = saved;
+    ctx->plan_chosen = chosen;
     ctx->plan_serial_ok = 1;
   }
-  const FinePlan batched = ctx->plan[0];
-  ctx->plan[0] = ctx->plan_serial;
   KD_LAUNCH(fill_slice_times(ctx->t0f, N + 1, 0, dT, ctx->st), "times");
   if ((s = copy_in_b0(ctx, b0)) != KD_OK) return s;
   for (int i = 0; i < N; ++i) {
@@ -1432,10 +1430,9 @@ kd_status kd_fine_serial(kd_ctx* ctx, const double* b0, double T, int N, double*
     KD_LAUNCH(compact_resample(KD_C128, ctx->U + 2 * i * len, n, pf, ctx->ws_f.X, n, 1, ctx->st), "to fine");
     FineArgs a = fine_args(ctx, ctx->ws_f, ctx->tab_f, n, 1, dt, ctx->t0f + i);
     if ((s = with_phases(ctx, ctx->ws_f, a, S)) != KD_OK) return s;
-    KD_LAUNCH(run_fine(ctx, 0, pf, a, S, true, false), "fine steps");
+    KD_LAUNCH(run_fine(ctx, 0, pf, a, S, true, false, nullptr, nullptr, &ctx->plan_serial), "fine steps");
     KD_LAUNCH(compact_resample(pf, ctx->ws_f.X, n, KD_C128, ctx->U + 2 * (i + 1) * len, n, 1, ctx->st), "from fine");
   }
-  ctx->plan[0] = batched;
   if ((s = copy_out_slices(ctx, u_slices, N)) != KD_OK) return s;
   KD_CUDA(cudaStreamSynchronize(ctx->st), "sync");
   return KD_OK;

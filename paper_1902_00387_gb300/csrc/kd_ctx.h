@@ -43,6 +43,7 @@ inline size_t csize(int prec) { return prec == KD_C128 ? 16 : 8; }
 struct kd_ctx {
   kd_params p;
   kd::FinePlan plan[2];        // launch plans of the fine (0) and coarse (1) grid
+  bool plan_chosen = false;    // plan[0] was set or tuned: calls of a few fields take it too (call_plan)
   kd::FinePlan plan_serial;    // fine-grid plan for one field at a time (kd_fine_serial)
   int plan_serial_ok = 0;
   int pdl = 1;                 // fine-step kernels as programmatic dependent launches
@@ -198,8 +199,8 @@ kd_status conv_fine(kd_ctx* ctx, const double* in, double* out, long batch, int 
 // fine steps on grid g (0 fine, 1 coarse) with the context's plan for that grid
 int run_fine(kd_ctx* ctx, int g, int prec, const kd::FineArgs& a, int nsteps, bool prologue, bool store_last,
              const kd::LaunchProbe* probe = nullptr, const int* active = nullptr, const kd::FinePlan* plan = nullptr);
-// fine-grid plan of a call over `batch` fields in all: the context's, or where that is the
-// default one the default for a few fields (fine_few); a call that works in chunks asks for the
+// fine-grid plan of a call over `batch` fields in all: the context's, or while nobody has chosen
+// one the default for a few fields (fine_few); a call that works in chunks asks for the
 // whole, so that its values do not depend on the chunks
 kd::FinePlan call_plan(const kd_ctx* ctx, long batch);
 

@@ -161,6 +161,13 @@ bool grid_of(kd_ctx* ctx, int grid, int* n, int* prec) {
   return true;
 }
 
+// The plan of a grid from now on, for calls of every batch.
+void choose(kd_ctx* ctx, int grid, int col, int row) {
+  ctx->plan[grid].col = col;
+  ctx->plan[grid].row = row;
+  if (grid == KD_GRID_FINE) ctx->plan_chosen = true;
+}
+
 }  // namespace
 
 extern "C" {
@@ -179,8 +186,7 @@ kd_status kd_set_plan(kd_ctx* ctx, int grid, int col, int row) {
   kd_status s = kd_plan_variants(ctx, grid, &nc, &nr);
   if (s != KD_OK) return s;
   if (col < 0 || col >= nc || row < 0 || row >= nr) return fail(ctx, KD_EINVAL, "kd_set_plan: variant out of range");
-  ctx->plan[grid].col = col;
-  ctx->plan[grid].row = row;
+  choose(ctx, grid, col, row);
   return KD_OK;
 }
 
@@ -253,8 +259,7 @@ kd_status kd_autotune(kd_ctx* ctx, int grid, int batch, int nsteps, const char* 
     for (const TuneEntry& e : cache)
       if (e.device == dev && e.n == n && e.prec == prec && e.batch == key && e.col >= 0 && e.col < nc && e.row >= 0 &&
           e.row < nr) {
-        ctx->plan[grid].col = e.col;
-        ctx->plan[grid].row = e.row;
+        choose(ctx, grid, e.col, e.row);
         if (ms_per_step) *ms_per_step = -1.0;
         return KD_OK;
       }
@@ -302,7 +307,7 @@ kd_status kd_autotune(kd_ctx* ctx, int grid, int batch, int nsteps, const char* 
     ctx->plan[grid] = saved;
     return s;
   }
-  ctx->plan[grid] = best_plan;
+  choose(ctx, grid, best_plan.col, best_plan.row);
   if (ms_per_step) *ms_per_step = best;
   if (cache_path) {
     TuneEntry e;

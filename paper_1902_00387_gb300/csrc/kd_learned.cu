@@ -533,42 +533,69 @@ int learned_momentum(float* W, const float* W0, const float* C2, float* v, __nv_
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
+// s + x = s' + err exactly (Knuth's two-sum)
+__device__ __forceinline__ void add_exact(float& s, float x, float& err) {
+  const float t = s + x, b = t - s;
+  err = (s - (t - b)) + (x - b);
+  s = t;
+}
+
 // The gradient grad = scale C2 + 2 wd (W - W0) of a caller's unpadded [rows][nc] matrices (C2: row
 // stride ldc) and, in the same pass, per-block sums of |W - W0|^2 (partials[2 b], [2 b + 1] = 0).
 // Bound by HBM: four matrices cross it once (1.66 GB at nc = 7203).  With the gradient, its
 // unpacking and the norm in passes of their own over padded copies of W and W0, and those copies
 // allocated and filled by each call, a call with 256 pairs took 8.0 ms; with this pass 2.1 (1.07 with
-// the operands' buffers kept between calls).  The norm is
-// summed as an unevaluated pair of floats a thread (differences, squares and sums with their
-// rounding errors, ~45 bits) and in FP64 across threads: an FP64 product and sum per element
-// would be bound by the few FP64 units.
+// the operands' buffers kept between calls).
+//
+// The norm is held to more than FP64's 53 bits without its units, whose few lanes an FP64 product
+// and sum per element would wait for: a thread sums the squares exactly split into floats, in a sum
+// of three floats (~70 bits) that loses only its third part's rounding; threads are added in FP64.
 __global__ void __launch_bounds__(TB) k_grad_norm(const float* W, const float* W0, const float* C2, int ldc,
                                                   float* grad, int rows, int nc, float scale, float wd,
                                                   double* partials) {
-  float sum = 0.f, low = 0.f;
+  constexpr int U = 4;                                       // tiles of TB columns of a row in flight
+  float s0 = 0.f, s1 = 0.f, s2 = 0.f;                        // the sum so far: s0 + s1 + s2
   double far = 0.0;
   const int chunks = (nc + TB - 1) / TB;
-  for (long t = blockIdx.x; t < (long)rows * chunks; t += gridDim.x) {
-    const int row = (int)(t / chunks), j = (int)(t - (long)row * chunks) * TB + threadIdx.x;
-    if (j >= nc) continue;
-    const long i = (long)row * nc + j;
-    const float w = W[i], w0 = W0 ? W0[i] : 0.f;
-    const float d = w - w0, bb = d - w;
-    const float dl = (w - (d - bb)) + (-w0 - bb);            // w - w0 = d + dl exactly
-    grad[i] = scale * C2[(long)row * ldc + j] + 2.f * wd * d;
-    const float p = __fmul_rn(d, d);
-    if (d == 0.f) continue;
-    if (!(p > 1e-24f && p < 1e30f)) {                        // no FP32 pair holds this square
-      const double e = (double)w - (double)w0;
-      far += e * e;
-      continue;
+  const long tiles = (long)rows * chunks;
+  for (long t0 = blockIdx.x; t0 < tiles; t0 += (long)U * gridDim.x) {
+    long at[U];
+    float w[U], w0[U], g[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const long t = t0 + (long)u * gridDim.x;
+      const int row = (int)(t / chunks), j = (int)(t - (long)row * chunks) * TB + threadIdx.x;
+      const bool in = t < tiles && j < nc;
+      at[u] = in ? (long)row * nc + j : -1;
+      w[u] = in ? W[at[u]] : 0.f;
+      w0[u] = in && W0 ? W0[at[u]] : 0.f;
+      g[u] = in ? C2[(long)row * ldc + j] : 0.f;
     }
-    const float pl = __fmaf_rn(2.f * d, dl, __fmaf_rn(d, d, -p));   // (w - w0)^2 = p + pl
-    const float s = sum + p, sb = s - sum;
-    low += ((sum - (s - sb)) + (p - sb)) + pl;
-    sum = s;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (at[u] < 0) continue;
+      const float d = w[u] - w0[u], bb = d - w[u];
+      const float dl = (w[u] - (d - bb)) + (-w0[u] - bb);    // w - w0 = d + dl exactly
+      grad[at[u]] = scale * g[u] + 2.f * wd * d;
+      const float p = __fmul_rn(d, d);
+      if (d == 0.f) continue;
+      if (!(p > 1e-24f && p < 1e30f)) {                      // no floats hold this square
+        const double x = (double)w[u] - (double)w0[u];
+        far += x * x;
+        continue;
+      }
+      // (w - w0)^2 = d d + 2 d dl + dl dl = (p + e) + (q + r), r rounded at 2^-71 of p
+      const float e = __fmaf_rn(d, d, -p), d2 = 2.f * d, q = __fmul_rn(d2, dl);
+      const float r = __fmaf_rn(dl, dl, __fmaf_rn(d2, dl, -q));
+      float a, b, c, f;
+      add_exact(s0, p, a);
+      add_exact(s1, a, b);
+      add_exact(s1, e, c);
+      add_exact(s1, q, f);
+      s2 += (b + c) + (f + r);
+    }
   }
-  block_sum2((double)sum + (double)low + far, 0.0, partials);
+  block_sum2((double)s0 + ((double)s1 + (double)s2) + far, 0.0, partials);
 }
 
 int learned_grad_norm(const float* W, const float* W0, const float* C2, int ldc, float* grad, int rows, int nc,

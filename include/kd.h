@@ -536,8 +536,9 @@ kd_status kd_block_get_state(kd_ctx* ctx, int local_index, double* u);
  * another scheme, means kernels on n points).  {0, 0} on every other grid.
  *
  * While no plan has been set or tuned, calls of a few fields in all take another default
- * at n = 256 (up to 6 fields: {0, 9}) and n = 512 (up to 3: {6, 9}), whose kernels spread
- * a field over the whole GPU.  Under one plan a field's values are the same bits in every
+ * at n = 256 (up to 4 fields: {0, 9}) and n = 512 (up to 2: {6, 9}), whose kernels spread
+ * a field over the whole GPU; the slices of a Parareal problem, the fields of a sweep's
+ * group and the pairs of kd_learned_pairs count as one call.  Under one plan a field's values are the same bits in every
  * batch; between two plans they differ by FP32 round-off.  A plan that was set or tuned is
  * the one that runs in every call, so setting the default keeps the bits of small batches.
  * grid: 0 = the fine grid n, 1 = the coarse grid n_coarse. */

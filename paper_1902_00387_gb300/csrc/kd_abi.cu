@@ -530,7 +530,7 @@ kd_status ensure_conv_tmp(kd_ctx* ctx, size_t bytes) {
 
 // Parallel fine step over slices [first, N): Fv[n] = F(U[n]), directly or in the
 // increment form Fv[n] += F(U[n] - Uprev[n]) (iter > 1).
-static kd_status fine_sweep_launches(kd_ctx* ctx, int first, int N, int S, double dt, int iter);
+static kd_status fine_sweep_launches(kd_ctx* ctx, int first, int N, int S, double dt, int iter, const FinePlan& plan);
 
 kd_status run_graph(kd_ctx* ctx, const std::string& key, const std::function<kd_status()>& launches) {
   // the graph runs on the context's own capturable stream, ordered after the work
@@ -573,11 +573,12 @@ kd_status run_graph(kd_ctx* ctx, const std::string& key, const std::function<kd_
 // The FFT operator's fine sweep is ~8 S + 3 launches; with graphs on, the launches of
 // one sweep shape are captured once into a CUDA graph (programmatic dependent launches
 // included) and replayed; the values are those of the direct launches.
-kd_status fine_sweep(kd_ctx* ctx, int first, int N, int S, double dt, int iter) {
+kd_status fine_sweep(kd_ctx* ctx, int first, int N, int S, double dt, int iter, long whole) {
+  const FinePlan plan = call_plan(ctx, whole);
   // (not for the pipelined iterations: their chunks already interleave with the serial
   // sweep on separate streams)
   if (!ctx->graphs || ctx->prof || ctx->overlap > 0 || conv_op(ctx) || N - first <= 0)
-    return fine_sweep_launches(ctx, first, N, S, dt, iter);
+    return fine_sweep_launches(ctx, first, N, S, dt, iter, plan);
   // the allocations the sweep may make happen before the capture
   {
     FineArgs a0 = fine_args(ctx, ctx->ws_f, ctx->tab_f, ctx->p.n, N - first, dt, ctx->t0f + first);
@@ -588,11 +589,12 @@ kd_status fine_sweep(kd_ctx* ctx, int first, int N, int S, double dt, int iter) 
   memcpy(&dbits, &dt, 8);
   char key[192];
   snprintf(key, sizeof(key), "parareal %d %d %d %lld %d %d %d %d %d %llu", first, N, S, dbits, iter == 1 ? 1 : 0,
-           ctx->plan[0].col, ctx->plan[0].row, ctx->pdl, ctx->p.fine_form, ctx->alloc_gen);
-  return run_graph(ctx, key, [&] { return fine_sweep_launches(ctx, first, N, S, dt, iter); });
+           plan.col, plan.row, ctx->pdl, ctx->p.fine_form, ctx->alloc_gen);
+  return run_graph(ctx, key, [&] { return fine_sweep_launches(ctx, first, N, S, dt, iter, plan); });
 }
 
-static kd_status fine_sweep_launches(kd_ctx* ctx, int first, int N, int S, double dt, int iter) {
+static kd_status fine_sweep_launches(kd_ctx* ctx, int first, int N, int S, double dt, int iter,
+                                     const FinePlan& plan) {
   const int n = ctx->p.n, pf = ctx->p.prec_fine;
   const long b = N - first;
   if (b <= 0) return KD_OK;
@@ -620,7 +622,7 @@ static kd_status fine_sweep_launches(kd_ctx* ctx, int first, int N, int S, doubl
   kd_status s = with_phases(ctx, ctx->ws_f, a, S);
   if (s != KD_OK) return s;
   LaunchProbe pr = probe_of(ctx);
-  KD_LAUNCH(run_fine(ctx, 0, pf, a, S, true, false, ctx->prof ? &pr : nullptr), "fine steps");
+  KD_LAUNCH(run_fine(ctx, 0, pf, a, S, true, false, ctx->prof ? &pr : nullptr, nullptr, &plan), "fine steps");
   if (incr)
     KD_LAUNCH(accum_out(pf, ctx->ws_f.X, ctx->Fv + 2 * first * len, b * len, iter == 1 ? 1 : 0, ctx->st),
               "accumulate fine");
@@ -703,7 +705,7 @@ kd_status pipelined_sweep(kd_ctx* ctx, int k, int N, int Sc, double dtc, const s
 
 // The fine chunks of iteration k on st2, each after its release event; records F per chunk
 // and the span events ts / te.
-kd_status pipelined_fine(kd_ctx* ctx, int k, int S, double dt, const std::vector<Chunk>& ck, cudaEvent_t ts,
+kd_status pipelined_fine(kd_ctx* ctx, int k, int N, int S, double dt, const std::vector<Chunk>& ck, cudaEvent_t ts,
                          cudaEvent_t te) {
   cudaEvent_t* E = &ctx->pev2[0];
   cudaEvent_t* F = &ctx->pev2[kMaxChunks];
@@ -717,7 +719,7 @@ kd_status pipelined_fine(kd_ctx* ctx, int k, int S, double dt, const std::vector
       s = cuda_fail(ctx, e, "fine chunk wait");
       break;
     }
-    s = fine_sweep(ctx, ck[j].lo, ck[j].hi, S, dt, k);
+    s = fine_sweep(ctx, ck[j].lo, ck[j].hi, S, dt, k, N);
     if (s == KD_OK && (e = cudaEventRecord(F[j], ctx->st2)) != cudaSuccess) s = cuda_fail(ctx, e, "fine chunk done");
   }
   if (s == KD_OK) {
@@ -753,7 +755,7 @@ kd_status parareal_pipelined(kd_ctx* ctx, int N, int S, int Sc, double dt, doubl
   KD_CUDA(cudaEventRecord(cs, ctx->st), "event");
   if ((s = pipelined_sweep(ctx, 0, N, Sc, dtc, {}, k_max >= 1 ? cur : std::vector<Chunk>())) != KD_OK) return s;
   KD_CUDA(cudaEventRecord(ce, ctx->st), "event");
-  if (k_max >= 1 && (s = pipelined_fine(ctx, 1, S, dt, cur, fs[1], fe[1])) != KD_OK) return s;
+  if (k_max >= 1 && (s = pipelined_fine(ctx, 1, N, S, dt, cur, fs[1], fe[1])) != KD_OK) return s;
   KD_CUDA(cudaEventSynchronize(ce), "sync");
   {
     float m0 = 0.f;
@@ -766,7 +768,7 @@ kd_status parareal_pipelined(kd_ctx* ctx, int N, int S, int Sc, double dt, doubl
     if ((s = pipelined_sweep(ctx, k, N, Sc, dtc, cur, next)) != KD_OK) return s;
     KD_CUDA(cudaMemcpyAsync(ctx->host_scal, ctx->scal, 8, cudaMemcpyDeviceToHost, ctx->st), "sigma copy");
     KD_CUDA(cudaEventRecord(ce, ctx->st), "event");
-    if (k < k_max && (s = pipelined_fine(ctx, k + 1, S, dt, next, fs[(k + 1) & 1], fe[(k + 1) & 1])) != KD_OK)
+    if (k < k_max && (s = pipelined_fine(ctx, k + 1, N, S, dt, next, fs[(k + 1) & 1], fe[(k + 1) & 1])) != KD_OK)
       return s;
     KD_CUDA(cudaEventSynchronize(ce), "sync");
     float m1 = 0.f, m2 = 0.f;
@@ -1279,7 +1281,7 @@ static kd_status parareal_core(kd_ctx* ctx, const double* b0, const double* u_in
     {
       NvtxRange rf("fine sweep");
       // the first iteration of a run, or of a resumed run, is in direct form
-      if ((s = fine_sweep(ctx, first, N, S, dt, (u_init && k == k0 + 1) ? 1 : k)) != KD_OK) return s;
+      if ((s = fine_sweep(ctx, first, N, S, dt, (u_init && k == k0 + 1) ? 1 : k, N)) != KD_OK) return s;
     }
     KD_CUDA(cudaEventRecord(ctx->ev[2], ctx->st), "event");
     NvtxRange rs("serial sweep");
@@ -1511,6 +1513,7 @@ kd_status kd_learned_pairs(kd_ctx* ctx, const float* x, int n, const int* phase,
   const int S = steps_for(ctx->l_sliceT, ctx->p.dt_fine);
   const double dt = ctx->l_sliceT / S;
   const int chunk = 512;
+  const FinePlan plan = call_plan(ctx, n);
   kd_status s;
   double* t0 = nullptr;
   if ((s = dalloc(ctx, (void**)&t0, chunk * 8, "times")) != KD_OK) return s;
@@ -1536,7 +1539,7 @@ kd_status kd_learned_pairs(kd_ctx* ctx, const float* x, int n, const int* phase,
     KD_LAUNCH(learned_to_fine(x + 2L * off * nc, K, P, ctx->ws_f.X, pf, Kf, Pf, cnt, ctx->st), "to fine");
     FineArgs a = fine_args(ctx, ctx->ws_f, ctx->tab_f, nfine, cnt, dt, t0);
     if ((s = with_phases(ctx, ctx->ws_f, a, S)) != KD_OK) return s;
-    KD_LAUNCH(run_fine(ctx, 0, pf, a, S, true, false), "fine steps");
+    KD_LAUNCH(run_fine(ctx, 0, pf, a, S, true, false, nullptr, nullptr, &plan), "fine steps");
     KD_LAUNCH(fine_to_learned(ctx->ws_f.X, pf, Kf, Pf, y + 2L * off * nc, K, P, cnt, ctx->st), "to learned");
     KD_CUDA(cudaStreamSynchronize(ctx->st), "sync");
   }

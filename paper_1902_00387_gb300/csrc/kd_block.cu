@@ -111,7 +111,7 @@ kd_status kd_block_fine(kd_ctx* ctx, int k) {
   if (has_last && first > ctx->blk_n - 1) first = ctx->blk_n - 1;
   if (first < 0) first = 0;
   if (first >= ctx->blk_n) return KD_OK;
-  if ((s = fine_sweep(ctx, first, ctx->blk_n, ctx->blk_S, ctx->blk_dt, k)) != KD_OK) return s;
+  if ((s = fine_sweep(ctx, first, ctx->blk_n, ctx->blk_S, ctx->blk_dt, k, ctx->blk_N)) != KD_OK) return s;
   KD_CUDA(cudaStreamSynchronize(ctx->st), "sync");
   return KD_OK;
 }

@@ -184,7 +184,9 @@ kd_status coarse_phases(kd_ctx* ctx, int N, int Sc, double dtc);
 kd_status coarse_step(kd_ctx* ctx, int i, int Sc, double dtc, bool init, bool last);
 kd_status learned_step(kd_ctx* ctx, int i, bool init, bool last);
 bool use_learned(const kd_ctx* ctx, int i);
-kd_status fine_sweep(kd_ctx* ctx, int first, int N, int S, double dt, int iter);
+// slices [first, N) of the context; whole: slices of the problem, over all ranks, chunks and
+// iterations, by which the launch plan is taken (call_plan)
+kd_status fine_sweep(kd_ctx* ctx, int first, int N, int S, double dt, int iter, long whole);
 // Enqueue `launches` (work on ctx->st) through a CUDA graph captured once per `key` and
 // replayed on the context's graph stream, fenced against ctx->st; the values are those of
 // the direct launches.  The caller makes every allocation the launches need beforehand

@@ -50,7 +50,9 @@ bool fine_variants(int n, int prec, int* ncol, int* nrow);
 // fine_few(n) fields (and for the coarse grid, whose serial sweep steps one at a time), which
 // leave most of the GPU idle in the default's larger blocks
 FinePlan fine_default_plan(int n, int prec, bool few = false);
-constexpr int fine_few(int n, int prec) { return prec != 0 ? 0 : (n == 256 ? 6 : (n == 512 ? 3 : 0)); }
+//   n = 256, (6, 0) | (0, 9), us a step of 1, 3, 4, 6 fields: 58.9 59.3 58.7 59.0 | 47.7 54.4 59.1 65.3
+//   n = 512, (5, 9) | (6, 9), of 1, 2, 3, 4 fields: 86.0 92.9 98.0 118.1 | 71.7 80.2 121.4 133.2
+constexpr int fine_few(int n, int prec) { return prec != 0 ? 0 : (n == 256 ? 4 : (n == 512 ? 2 : 0)); }
 // Row variant of the warp-transform row kernel of the complex64 n = 1024 grid
 constexpr int kRow4Variant = 7;
 // whether the plan's kernels read the first step's state from FineArgs::x_in_full and

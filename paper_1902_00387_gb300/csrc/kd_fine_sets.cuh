@@ -294,7 +294,7 @@ struct Fine2Set {
   static int nrow() { return nrow0() + (MR ? 1 : 0) + (WT ? 1 : 0); }
   // plan of a context that is not autotuned: the persistent fused step; for one field at a time
   // (few) at n = 256 the warp-transform row kernel with the four-step column kernel, which spread
-  // a field over the whole GPU instead of 16 SMs (47 us a step against 59; 8 fields: 80 and 78)
+  // a field over the whole GPU instead of 16 SMs (both measured at fine_few)
   static FinePlan default_plan(bool few) {
     FinePlan p;
     if (few && WT && N == 256)
@@ -435,9 +435,8 @@ struct Fine3Set {
     return scheme == SCHEME_RK443 && ((W4 && col == kW6Col && row == kW4Row) || (R8 && col == kC512Col && row == kC512Row));
   }
   static int ncol() { return WIDE ? (R8 ? 7 : (W4 ? 7 : 4)) : 1; }
-  // plan of a context that is not autotuned: the 3n/4-point pairs; for up to three fields of
-  // 512^2 (few) the 512-point warp kernels, whose blocks are smaller (1, 2, 4 fields: 72, 80,
-  // 133 us a step against 88, 97, 132)
+  // plan of a context that is not autotuned: the 3n/4-point pairs; for a few fields of
+  // 512^2 the 512-point warp kernels, whose blocks are smaller (both measured at fine_few)
   static FinePlan default_plan(bool few) {
     FinePlan p;
     if (W4) {

@@ -307,11 +307,12 @@ kd_status exec_group(kd_ctx* ctx, std::vector<Member>& mem, GroupBufs& g, double
       a.flow = KD_FLOW_GALLOWAY_PROCTOR;   // the phase table holds every field's flow
       a.sp = g.spf;
       if ((s = with_phases(ctx, ctx->ws_f, a, Smax)) != KD_OK) return s;
+      const FinePlan plan = call_plan(ctx, (long)m * N);   // by the group, whatever is still active
       auto launches = [&]() -> kd_status {
         k_delta_in_map<float><<<grid1(nE * len), 256, 0, ctx->st>>>((const cx<double>*)g.U, (cx<double>*)g.Up,
                                                                       (cx<float>*)ctx->ws_f.X, g.emap, len, nE, k == 1);
         KD_LAUNCH(0, "increment to fine");
-        KD_LAUNCH(run_fine(ctx, 0, KD_C64, a, Smax, true, false, nullptr, act_f.data()), "fine steps");
+        KD_LAUNCH(run_fine(ctx, 0, KD_C64, a, Smax, true, false, nullptr, act_f.data(), &plan), "fine steps");
         k_accum_out_map<float><<<grid1(nE * len), 256, 0, ctx->st>>>((const cx<float>*)ctx->ws_f.X,
                                                                        (cx<double>*)g.Fv, g.emap, len, nE, k == 1);
         KD_LAUNCH(0, "accumulate fine");
@@ -321,8 +322,8 @@ kd_status exec_group(kd_ctx* ctx, std::vector<Member>& mem, GroupBufs& g, double
         // replayed when the same (iteration, active members, plan) recurs, e.g. in a
         // repeated kd_sweep_exec of the same instances
         std::string key = "sweep " + std::to_string(k == 1) + " " + std::to_string(first) + " " +
-                          std::to_string(nE) + " " + std::to_string(Smax) + " " + std::to_string(ctx->plan[0].col) +
-                          "," + std::to_string(ctx->plan[0].row) + " " + std::to_string(ctx->pdl) + " " +
+                          std::to_string(nE) + " " + std::to_string(Smax) + " " + std::to_string(plan.col) +
+                          "," + std::to_string(plan.row) + " " + std::to_string(ctx->pdl) + " " +
                           std::to_string(ctx->alloc_gen) + " :";
         for (int r : Af) key += " " + std::to_string(r);
         if ((s = run_graph(ctx, key, launches)) != KD_OK) return s;

@@ -27,8 +27,9 @@
 //                     9 = 512-point warp transforms, one warp per component of a row
 //                     (kd_fine5.cuh; n = 512)
 //   n = 1024  column: 4 = warp-owned transforms (kd_fine4.cuh), one warp per component,
-//                     4 columns per block; 5, 6 = warp-owned transforms, one warp per column,
-//                     8 columns per block
+//                     4 columns per block; 5 = warp-owned transforms, one warp per column,
+//                     8 columns per block; 6 = the same with two independent groups of
+//                     4 columns per block
 //             row:    7 = warp-owned transforms, one row per block
 //   The default pairs (column 6, row 7) at n = 1024 and (5, 9) at n = 512 step RK443 on 3n/4
 //   points with the kernels of kd_narrow.cuh (the two kernels of a plan share the mixed
@@ -349,7 +350,9 @@ struct Fine2Set {
     if constexpr (R8) {
       if (v == 3) return launch_col3<T, N, Shapes8<N>::XT, 8>(a, s, j, st, pdl);
     }
-    if (WIDE && v == 1)
+    // the fused step's variant at a scheme it does not have: the faster tile shape for these (n = 128:
+    // xt(1), RK222 us a step of 1 and 100 fields 53 and 161 against 56 and 167)
+    if (WIDE && (v == 1 || (N == 128 && v == fused_col(N))))
       launch_col2<T, N, Sh::xt(1)>(a, s, j, st, pdl);
     else
       launch_col2<T, N, Sh::xt(0)>(a, s, j, st, pdl);
@@ -464,6 +467,9 @@ struct Fine3Set {
       if ((e = cudaFuncSetAttribute(col5_kernel<N, 8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)Col5<N, 8, 1>::smem)) != cudaSuccess)
         return e;
+      if ((e = cudaFuncSetAttribute(col5_kernel<N, 4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)Col5<N, 4, 2>::smem)) != cudaSuccess)
+        return e;
       if ((e = prepare_row4<N, 0>()) != cudaSuccess) return e;
       if ((e = prepare_row4<N, 1>()) != cudaSuccess) return e;
       if ((e = prepare_row4<N, 2>()) != cudaSuccess) return e;
@@ -509,10 +515,16 @@ struct Fine3Set {
       if (v == kNarrowVariant) return launch_coln<NN>(a, s, j, st, pdl);
     }
     if constexpr (W4) {
-      if (v == kW5Col || v == kW6Col) {
+      if (v == kW5Col) {
         using C5 = Col5<N, 8, 1>;
         launch_k(col5_kernel<N, 8, 1>, persistent_grid((long)a.batch * (N / C5::XG)), C5::BLOCK, C5::smem, st, pdl,
                  a, s, j);
+        return;
+      }
+      if (v == kW6Col) {
+        using C6 = Col5<N, 4, 2>;
+        const long groups = (long)a.batch * (N / C6::XG);
+        launch_k(col5_kernel<N, 4, 2>, persistent_grid((groups + 1) / 2), C6::BLOCK, C6::smem, st, pdl, a, s, j);
         return;
       }
       if (v == kW4Col) {

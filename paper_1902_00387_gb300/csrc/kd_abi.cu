@@ -196,7 +196,14 @@ kd_status ensure_ws(kd_ctx* ctx, FineWs& w, int n, int prec, long batch) {
   // complex64 state: its low part within a propagation call (kd_stage.cuh)
   if (prec == KD_C64 && (s = dalloc(ctx, &w.Xlo, spec, "state low part")) != KD_OK) return s;
   if ((s = dalloc(ctx, &w.M, mixed, "mixed M")) != KD_OK) return s;
-  if ((s = dalloc(ctx, &w.W, mixed, "mixed W")) != KD_OK) return s;
+  // room for the launches of a few fields where there is any (they step in clusters without it)
+  const size_t wide = (size_t)fused_spread_len(n / 3, prec, batch) * es;
+  if (wide > mixed && dalloc(ctx, &w.W, wide, "mixed W") == KD_OK)
+    w.w_len = (long)(wide / es);
+  else if ((s = dalloc(ctx, &w.W, mixed, "mixed W")) != KD_OK)
+    return s;
+  else
+    w.w_len = (long)(mixed / es);
   w.cap = batch;
   w.n = n;
   w.prec = prec;
@@ -224,6 +231,7 @@ FineArgs fine_args(const kd_ctx* ctx, const FineWs& w, const Tables& t, int n, l
   a.lo_valid = 0;
   a.M = w.M;
   a.W = w.W;
+  a.w_len = w.w_len;
   a.tw = t.tw;
   a.cosg = t.cosg;
   a.sing = t.sing;

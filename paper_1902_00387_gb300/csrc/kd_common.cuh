@@ -86,6 +86,7 @@ struct FineArgs {
   int lo_valid;      // Xlo holds the low part of X (false before the first step of a call)
   void* M;           // mixed (inverse-x) field     [batch][3][P][n]
   void* W;           // mixed (forward-y) product   [batch][3][P][n]
+  long w_len = 0;    // complex values that W holds (fused_spread_len; 0: those of its own layout)
   const void* tw;
   const void* cosg;
   const void* sing;

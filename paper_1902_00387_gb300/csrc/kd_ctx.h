@@ -32,6 +32,7 @@ struct FineWs {
   void* Xlo = nullptr;     // complex64: low part of the state within a propagation call
   void* M = nullptr;
   void* W = nullptr;
+  long w_len = 0;          // complex values that W holds
   void* ph = nullptr;      // flow-phase table
   size_t ph_bytes = 0;
 };

@@ -73,6 +73,12 @@ cudaError_t fused_prepare(int prec, int K);   // the kernel of the kept set K (0
 // Enqueue cfg.nsteps steps from a.X to a.X (a.phases filled); returns the kernels launched,
 // negative on failure.  Needs a prologue call that keeps no mixed field.
 int fused_run(int prec, const FineArgs& a, const StepCfg& cfg);
+// Fields up to which the passes of a complex128 kept set on 192 points (K = 64..95) run as launches
+// over the whole GPU (kd_fused.cu), and the complex values of FineArgs::W that these take (0: other sets)
+constexpr int kSpreadFields = 24;
+inline long fused_spread_len(int K, int prec, long batch) {
+  return prec != 0 && K >= 64 && K <= 95 ? 3L * (2 * K + 1) * 192 * (batch < kSpreadFields ? batch : kSpreadFields) : 0;
+}
 // column variant of the complex64 sides 16..256 that selects it
 constexpr int fused_col(int n) { return n == 128 ? 4 : (n == 256 ? 6 : (n == 16 ? 3 : 4)); }
 

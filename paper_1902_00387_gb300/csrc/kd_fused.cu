@@ -14,11 +14,22 @@ constexpr int kShapes[] = {1, 2, 3, 4, 6, 8, 12, 16};   // blocks a cluster
 constexpr int kNShapes = 8;
 constexpr size_t kMaxSmem = 232448;                     // shared memory a block may opt in to
 
+template <typename T, int L, int R>
+int run_spread(const FineArgs& a, const StepCfg& cfg, int s, int e);
+
 // A kernel with the threads (0: the shape does not fit) and shared memory of its blocks.
 template <typename T, int L, int R>
 struct LaneKernel {
   using F = FusedStep<T, L, R>;
   static constexpr auto kernel = fused_kernel<T, L, R>;
+  // Fields for which the passes run as launches of their own (0: never).  An SM has few FP64 units
+  // and a field has 16 SMs at most in a cluster, so that up to nine fields take what one takes.  192^2
+  // complex128, us a step of 1, 4, 8, 12, 24 fields, clusters | launches: 1070 1072 1323 2071 4131 |
+  // 640 776 1007 1334 2616.  More fields gain less (40: 4934 | 4140), for room in W that grows with them.
+  // In complex64 the launches' latencies take what the units would give (54 55 75 88 141 | 49 56 81
+  // 114 198).
+  static constexpr int SPREAD = L * R == 192 && sizeof(T) == 8 ? kSpreadFields : 0;
+  static int spread(const FineArgs& a, const StepCfg& cfg, int s, int e) { return run_spread<T, L, R>(a, cfg, s, e); }
   static int threads(int P, int CS) { return F::N % CS == 0 && F::smem(P, CS) <= kMaxSmem ? 32 * F::warps(P, CS) : 0; }
   static size_t smem(int P, int CS) { return F::smem(P, CS); }
 };
@@ -63,6 +74,29 @@ int active_clusters(int P, int shape) {
   }
   if (dev < 16) cache[dev][K][shape] = (short)(n < 32000 ? n + 1 : 32000);
   return n;
+}
+
+// Steps [s, e) of the fields of a, a launch a pass (fused_kernel); returns the launches, negative on failure.
+template <typename T, int L, int R>
+int run_spread(const FineArgs& a, const StepCfg& cfg, int s, int e) {
+  constexpr int N = L * R;
+  cudaLaunchAttribute at[2];
+  auto pass = [&](int kid, int tasks, auto kernel, size_t smem, int step, int stage, bool more) {
+    cudaLaunchConfig_t lc = config(1, 1, 32, smem, cfg.st, cfg.pdl, at);
+    lc.gridDim = dim3((unsigned)tasks, (unsigned)a.batch, 1);
+    if (cfg.probe) cfg.probe->before(cfg.probe->user, kid);
+    if (cudaLaunchKernelEx(&lc, kernel, a, (int)more, step, stage) != cudaSuccess) return false;
+    if (cfg.probe) cfg.probe->after(cfg.probe->user, kid);
+    return true;
+  };
+  auto cols = fused_kernel<T, L, R, FUSED_COLS>;
+  auto rows = fused_kernel<T, L, R, FUSED_ROWS>;
+  if (!pass(1, a.P, rows, 0, s, 4, true)) return -1;
+  for (int st = s; st < e; ++st)
+    for (int j = 0; j < 4; ++j)
+      if (!pass(0, N, cols, N * sizeof(cx<T>), st, j, true) || !pass(1, a.P, rows, 0, st, j, st + 1 < e || j < 3))
+        return -1;
+  return 1 + 8 * (e - s);
 }
 
 // Blocks a cluster for a batch: the shape with the least waves (co / CS + 1/8 + co CS / 400), co
@@ -112,6 +146,15 @@ int run_one(const FineArgs& a0, const StepCfg& cfg) {
       e = s + 1;
       while (e < cfg.nsteps && cfg.active[e] == a.batch) ++e;
     }
+    if constexpr (KT::SPREAD > 0) {
+      if (a.batch <= KT::SPREAD && a.w_len >= 3L * a.P * KT::F::N * a.batch) {
+        const int r = KT::spread(a, cfg, s, e);
+        if (r < 0) return -1;
+        launches += r;
+        s = e;
+        continue;
+      }
+    }
     const int CS = shape_for<KT>(a.P, a.batch);
     if (CS == 0) return -1;
     cudaLaunchAttribute at[2];
@@ -126,13 +169,15 @@ int run_one(const FineArgs& a0, const StepCfg& cfg) {
 }
 
 // f(kernel) for the kernel of the kept set K: the smallest N >= 2K + 2 points.  complex128 takes
-// 32 x 1 instead of 8 x 3 points for the smallest sets: an FP64 instruction costs an SM's quarter
-// 64 cycles whatever its lanes do, so a third of the values a lane is a third of the time for the
-// few fields of such a grid (8 fields of 32^2: 57 us a step against 142).
+// 16 x 1 and 32 x 1 instead of 8 x 3 points for the smallest sets: an FP64 instruction costs an SM's
+// quarter 64 cycles whatever its lanes do, so a third of the values a lane is a third of the time for
+// the few fields of such a grid (8 fields of 32^2: 57 us a step against 142; 16^2 on 16 | 32 points: 1
+// field 46 | 57, 100 59 | 201, 300 131 | 459, which the kernels of kd_fine2.cuh take in 129, 145, 198).
 template <typename T, class Fn>
 auto with_kernel(int K, Fn&& f) {
   const int m = 2 * K + 2;
   if constexpr (sizeof(T) == 8) {
+    if (m <= 16) return f(LaneKernel<T, 16, 1>());
     if (m <= 32) return f(LaneKernel<T, 32, 1>());
   } else {
     if (m <= 24) return f(LaneKernel<T, 8, 3>());
@@ -147,7 +192,7 @@ template <typename T>
 cudaError_t prepare_T(int K) {
   auto prep = [](auto k) { return prepare_one<decltype(k)>(); };
   if (K > 0) return 2 * K + 2 <= 192 ? with_kernel<T>(K, prep) : cudaSuccess;
-  for (int k : {5, 20, 40, 60, 90}) {
+  for (int k : {5, 10, 20, 40, 60, 90}) {
     const cudaError_t e = with_kernel<T>(k, prep);
     if (e != cudaSuccess) return e;
   }

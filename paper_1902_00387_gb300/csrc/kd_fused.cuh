@@ -305,30 +305,42 @@ __device__ __forceinline__ cx<T> fused_update(cx<T>* o0, cx<T>* o1, cx<T>* o2, b
   }
 }
 
-// Steps [s0, s0 + nsteps) of every field b = blockIdx.x / CS, from the state X (and Xlo when
-// s0 > 0) back to X (Xlo).
-template <typename T, int L, int R>
-__global__ void __launch_bounds__(32 * FusedStep<T, L, R>::MAXW, 1) fused_kernel(FineArgs a, int CS, int s0, int nsteps) {
+// FUSED_CLUSTER: steps [s0, s0 + nsteps) of every field b = blockIdx.x / CS, from the state X (and
+// Xlo when s0 > 0) back to X (Xlo).
+//
+// A few fields of the largest complex128 sets leave most of the GPU idle in clusters, 16 SMs each at
+// most.  For them (LaneKernel::SPREAD in kd_fused.cu) the same passes run as launches over the whole GPU, a warp a block, with the mixed field in global memory (a.W, L2):
+// FUSED_COLS: column pass of stage nsteps of step s0, field blockIdx.y; FUSED_ROWS: row pass (4:
+// before the first stage), CS: whether another stage follows.  The arithmetic is this one source's,
+// so the values are the same bits.
+enum { FUSED_CLUSTER = 0, FUSED_COLS = 1, FUSED_ROWS = 2 };
+
+template <typename T, int L, int R, int MODE = FUSED_CLUSTER>
+__global__ void __launch_bounds__(MODE == FUSED_CLUSTER ? 32 * FusedStep<T, L, R>::MAXW : 32, 1)
+    fused_kernel(FineArgs a, int CS, int s0, int nsteps) {
   using F = FusedStep<T, L, R>;
+  constexpr bool CL = MODE == FUSED_CLUSTER;
   constexpr int N = F::N, TPW = F::TPW;
   // registers of the row whose stage arrays are in flight ahead of their use
   constexpr int AHEAD = sizeof(T) == 4 ? (R == 6 ? 3 : R) : (R == 1 ? 1 : 2);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int K = a.K, P = a.P;
-  const int XH = N / CS, XP = F::xp(XH), RH = (P + CS - 1) / CS;
-  const int rank = (int)(blockIdx.x % CS);
-  const long b = blockIdx.x / CS;
+  const int XH = CL ? N / CS : N, XP = CL ? F::xp(XH) : N, RH = CL ? (P + CS - 1) / CS : P;
+  const int rank = CL ? (int)(blockIdx.x % CS) : 0;
+  const long b = CL ? blockIdx.x / CS : blockIdx.y;
   const int x0 = rank * XH, y0 = rank * RH, rows = max(0, min(RH, P - y0));
   // the warp index as the uniform value that it is: the loops over a warp's tasks then need no
   // re-convergence before each shuffle (a third of the instructions otherwise)
-  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), nw = blockDim.x >> 5;
+  const int warp = CL ? __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0) : blockIdx.x;
+  const int nw = CL ? blockDim.x >> 5 : gridDim.x;
   const int l = threadIdx.x & (L - 1), grp = (threadIdx.x & 31) / L;   // lane and transform of the warp's TPW
-  cx<T>* B = (cx<T>*)smem_raw;                     // [3][P][XP]
-  cx<T>* s_cs = B + F::field(P, CS);               // (cos, sin)(2 pi j / N)
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    const cx<T> w = wt_tw<N, T>(i);
-    s_cs[i] = mk(w.x, -w.y);
-  }
+  cx<T>* B = CL ? (cx<T>*)smem_raw : (cx<T>*)a.W + b * 3 * P * N;   // [3][P][XP]
+  cx<T>* s_cs = CL ? B + F::field(P, CS) : (cx<T>*)smem_raw;        // (cos, sin)(2 pi j / N)
+  if (MODE != FUSED_ROWS)
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+      const cx<T> w = wt_tw<N, T>(i);
+      s_cs[i] = mk(w.x, -w.y);
+    }
   const LaneFFT<T, L, R> fft(l);
   const StageCoef<T> sc = stage_coef<T>(a, b);
   const T A = flow_amp<T>(a, b);
@@ -357,10 +369,12 @@ __global__ void __launch_bounds__(32 * FusedStep<T, L, R>::MAXW, 1) fused_kernel
       kx_on[k] = i <= K || i >= N - K;
       slot[k] = first + (i <= K ? m : nlow + m - mhigh);
       first += nlow + L - mhigh;
-      const int x = l + L * k, own = x / XH;
-      near[k] = own == rank;
-      at_q[k] = (uint32_t)__cvta_generic_to_shared(B + x - own * XH);
-      if (!near[k]) at_q[k] = fused_peer(at_q[k], own);
+      if (CL) {
+        const int x = l + L * k, own = x / XH;
+        near[k] = own == rank;
+        at_q[k] = (uint32_t)__cvta_generic_to_shared(B + x - own * XH);
+        if (!near[k]) at_q[k] = fused_peer(at_q[k], own);
+      }
     }
   }
   const uint32_t row_b = (uint32_t)(XP * (int)sizeof(cx<T>));   // bytes of a row of B
@@ -398,7 +412,8 @@ __global__ void __launch_bounds__(32 * FusedStep<T, L, R>::MAXW, 1) fused_kernel
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
-          for (int q = 0; q < R; ++q) v[c][q] = fused_ld(at_q[q] + (uint32_t)(c * P + iy) * row_b, near[q], T(0));
+          for (int q = 0; q < R; ++q)
+            v[c][q] = CL ? fused_ld(at_q[q] + (uint32_t)(c * P + iy) * row_b, near[q], T(0)) : B[(c * P + iy) * N + l + L * q];
         fft.template a_to_b<-1>(v);                // x -> kx
         const T fky = (T)(iy - K), kz = sc.kz, ly = fky * fky + kz * kz;
         auto update = [&](auto mode_c) {
@@ -444,7 +459,11 @@ __global__ void __launch_bounds__(32 * FusedStep<T, L, R>::MAXW, 1) fused_kernel
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
-          for (int q = 0; q < R; ++q) fused_st(at_q[q] + (uint32_t)(c * P + iy) * row_b, near[q], v[c][q]);
+          for (int q = 0; q < R; ++q)
+            if (CL)
+              fused_st(at_q[q] + (uint32_t)(c * P + iy) * row_b, near[q], v[c][q]);
+            else
+              B[(c * P + iy) * N + l + L * q] = v[c][q];
       }
     }
   };
@@ -490,18 +509,28 @@ __global__ void __launch_bounds__(32 * FusedStep<T, L, R>::MAXW, 1) fused_kernel
     }
   };
 
-  griddep_wait();                                  // X comes from the predecessor
-  fused_cluster_sync();                            // tables; every block of the cluster runs
-  // one copy of each pass: the prologue is the row pass before the first stage
+  if constexpr (CL) {
+    griddep_wait();                                // X comes from the predecessor
+    fused_cluster_sync();                          // tables; every block of the cluster runs
+    // one copy of each pass: the prologue is the row pass before the first stage
 #pragma unroll 1
-  for (int it = -1; it < 4 * nsteps; ++it) {
-    const int s = s0 + (it >> 2), j = it & 3;
-    if (it >= 0) {
-      col_pass(s, j);
-      fused_cluster_sync();
+    for (int it = -1; it < 4 * nsteps; ++it) {
+      const int s = s0 + (it >> 2), j = it & 3;
+      if (it >= 0) {
+        col_pass(s, j);
+        fused_cluster_sync();
+      }
+      row_pass(it < 0 ? 4 : j, it + 1 < 4 * nsteps, s > 0);
+      fused_cluster_sync();   // B is complete; after the last stage: no peer reads it any more
     }
-    row_pass(it < 0 ? 4 : j, it + 1 < 4 * nsteps, s > 0);
-    fused_cluster_sync();   // B is complete; after the last stage: no peer reads it any more
+  } else {
+    griddep_launch_dependents();                   // the next pass waits for this one's end itself
+    __syncwarp();                                  // table
+    griddep_wait();
+    if constexpr (MODE == FUSED_COLS)
+      col_pass(s0, nsteps);
+    else
+      row_pass(nsteps, CS != 0, s0 > 0);
   }
 }
 

@@ -477,9 +477,12 @@ kd_status kd_selftest_wait(int arrive, double max_ms, void* cuda_stream);
  * tables, fine and coarse workspaces, Parareal arrays, staging; not CUDA's own objects
  * such as streams, events and graph executables, nor the static array of
  * kd_fine_batched_static).  Training buffers that the context keeps for its next training
- * call (at most 1 GiB) count as held and are released before a request is refused or, on a
- * GPU that is out of memory, fails.  max_bytes = 0 removes it (the default); a limit below what the
- * context already holds keeps those buffers and refuses new ones.  A call that needs a
+ * call (at most 1 GiB, the newest) count as held and are released
+ * before a request is refused; on a GPU that is out of memory those of every context are
+ * released before a request of any fails.  Other allocators of the process (PyTorch) cannot
+ * ask for them: kd_destroy gives a context's back.  max_bytes = 0 removes the limit (the
+ * default); a limit below what the context already holds keeps the buffers in use and
+ * refuses new ones.  A call that needs a
  * buffer beyond the limit returns KD_ENOMEM, as a failed cudaMalloc does, with
  * kd_last_error naming the buffer, its size, the bytes held and the limit; the context
  * stays usable, and the same call succeeds once the limit allows it.  Contexts that

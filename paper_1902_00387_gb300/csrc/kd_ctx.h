@@ -108,8 +108,6 @@ struct kd_ctx {
   std::vector<size_t> alloc_sizes;
   size_t alloc_held = 0;
   size_t alloc_limit = 0;
-  std::vector<size_t> spare;  // entries of allocs that dkeep released, oldest first
-  size_t spare_bytes = 0;
   std::string err;
   long long launches = 0;     // kernels launched by this context
   int cK = 0, cP = 0;         // coarse mode set k in [-cK, cP - cK)^2

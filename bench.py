@@ -279,16 +279,28 @@ class ClockSampler:
 
 
 # ---------------------------------------------------------------- roofline
-def col_row_bytes(n, batch_slices):
-    """Algorithmic bytes of one column launch and of one row launch (complex64):
-    the column pass reads and writes the mixed field (3 x P x N); the row pass reads
-    and writes it too and touches compact spectral arrays (3 x P x P) over the four
-    stages.  Sides 512 and 1024 work on N = 3n/4 points and move 2, 4, 3, 3 compact
-    arrays at the stages (the state; its low part is not counted), the two-kernel step
-    of the other sides on N = n with 4, 5, 3, 2."""
+# launch plans (kd_get_plan) of the complex64 RK443 step: the column variant of the persistent step
+# and the pairs that step on 3n/4 points
+PERSISTENT_COL = {16: 3, 32: 4, 64: 4, 128: 4, 256: 6}
+NARROW_PLAN = {512: (5, 9), 1024: (6, 7)}
+
+
+def persistent(n, plan):
+    """Whether complex64 RK443 steps of side n run in the persistent kernel under the plan (the
+    sides that are no powers of two have one plan)."""
+    return PERSISTENT_COL[n] == plan[0] if n in PERSISTENT_COL else n <= 286
+
+
+def col_row_bytes(n, batch_slices, plan):
+    """Algorithmic bytes of one column launch and of one row launch (complex64) of a
+    two-kernel step under the plan: the column pass reads and writes the mixed field
+    (3 x P x N); the row pass reads and writes it too and touches compact spectral arrays
+    (3 x P x P) over the four stages.  The 3n/4-point pairs of 512 and 1024 work on N = 3n/4
+    points and move 2, 4, 3, 3 compact arrays at the stages (the state; its low part is not
+    counted), the other plans on N = n with 4, 5, 3, 2."""
     K = n // 3
     P = 2 * K + 1
-    narrow = n in (512, 1024)
+    narrow = NARROW_PLAN.get(n) == tuple(plan)
     mixed = 3 * P * (3 * n // 4 if narrow else n) * 8
     spec = 3 * P * P * 8
     return 2 * mixed * batch_slices, (2 * mixed + (3.0 if narrow else 3.5) * spec) * batch_slices
@@ -302,6 +314,23 @@ def fused_bytes(n, batch_slices):
     compact arrays of the four stages; the mixed field stays in shared memory."""
     P = 2 * (n // 3) + 1
     return FUSED_PASSES * 3 * P * P * 8 * batch_slices
+
+
+def step_bytes_of(n, batch_slices, plan):
+    """Algorithmic bytes of one complex64 RK443 step of the fields under the plan."""
+    if persistent(n, plan):
+        return fused_bytes(n, batch_slices)
+    return 4 * sum(col_row_bytes(n, batch_slices, plan))
+
+
+def tuned_plan(cache, device, n, batch):
+    """The complex64 plan of a tuning file (kd_autotune) for side n and a batch."""
+    key = 1 << (batch - 1).bit_length()
+    with open(cache) as f:
+        for e in json.load(f)["entries"]:
+            if (e["device"], e["n"], e["prec"], e["batch"]) == (device, n, 0, key):
+                return e["col"], e["row"]
+    raise RuntimeError("no plan of side %d for %d fields in %s" % (n, batch, cache))
 
 
 # --------------------------------------------------- learned coarse propagator run
@@ -748,7 +777,7 @@ def run_large(args):
     kd.kd_fine_batched(ctx, x, x, t0, 2, N)
     prof_ms, prof_n = kd.kd_profile_read(ctx)
     kd.kd_profile(ctx, 0)
-    cb, rb = col_row_bytes(n, N)
+    cb, rb = col_row_bytes(n, N, plan_f)
     step_bytes = 4 * (cb + rb)
     achieved = (cb * prof_n[0] + rb * prof_n[1]) / ((prof_ms[0] + prof_ms[1]) / 1e3) / 1e9
     kid = 0 if prof_ms[0] >= prof_ms[1] else 1
@@ -872,12 +901,18 @@ def run_sweep(args):
     # serial-fine-equivalent work of one solve: every instance's N x S fine steps
     units = sum(3 * q.n ** 2 * N * r.n_fine_steps for q, r in zip(ins, results))
     value = units * world * args.steps / el / 1e6
-    # fine work actually done and its two-pass algorithmic bytes
+    # fine work actually done and its algorithmic bytes under the plan of each side's group
+    sides = sorted({q.n for q in ins})
+    device = torch.cuda.get_device_name()
+    plans = {n: tuned_plan(cache, device, n, N * sum(1 for q in ins if q.n == n)) for n in sides}
     fine_bytes = 0.0
     for q, r in zip(ins, results):
-        cb, rb = col_row_bytes(q.n, 1)
-        per_slice_step = 4 * (cb + rb)
+        per_slice_step = step_bytes_of(q.n, 1, plans[q.n])
         fine_bytes += sum(N - min(k - 1, N - 1) for k in range(1, r.k_con + 1)) * r.n_fine_steps * per_slice_step
+    one_launch = [n for n in sides if persistent(n, plans[n])]
+    two = [n for n in sides if n not in one_launch]
+    kernels = ["%s at %s" % (k, ", ".join(map(str, v))) for k, v in
+               (("persistent step", one_launch), ("column + row kernels", two)) if v]
     hbm_peak, peak_kind = peaks()
     achieved = fine_bytes / (st.ms_fine / 1e3) / 1e9
     e2e_value = None
@@ -901,7 +936,10 @@ def run_sweep(args):
         "converged": sum(1 for r in results if r.status == kd.KD_OK), "k_con_max": max(ks),
         "phase_ms": {"fine": st.ms_fine, "coarse_and_update": st.ms_coarse, "total": st.ms_total},
         "fine_mdof_steps_per_s": st.fine_dof_steps / (st.ms_fine / 1e3) / 1e6,
-        "roofline": {"bound": "hbm", "kernel": "fine phase (column + row kernels, increment gather/scatter)",
+        "fine_plans": {str(n): list(p) for n, p in plans.items()},
+        "roofline": {"bound": "hbm" if not one_launch else "issue and latency (persistent step, L2-resident)" if not two
+                     else "issue and latency (persistent step, L2-resident); hbm (column + row kernels)",
+                     "kernel": "fine phase (%s; increment gather/scatter)" % "; ".join(kernels),
                      "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
                      "traffic": None, "peak_kind": peak_kind},
         "clocks": clk,
@@ -1092,8 +1130,8 @@ def parareal_c2(args, env, embedded):
     # fine-sweep batches over one solve: slices k-1..N-1 in iteration k
     batches = [N - min(k - 1, N - 1) for k in range(1, st.k_con + 1)]
     fused = prof_n[0] == 0 and prof_n[1] > 0     # the persistent step: one launch a sweep, all its steps
-    col_b = sum(col_row_bytes(n, b)[0] * 4 * S for b in batches) * prof_steps
-    row_b = sum((fused_bytes(n, b) if fused else col_row_bytes(n, b)[1] * 4) * S for b in batches) * prof_steps
+    col_b = sum(col_row_bytes(n, b, plan)[0] * 4 * S for b in batches) * prof_steps
+    row_b = sum((fused_bytes(n, b) if fused else col_row_bytes(n, b, plan)[1] * 4) * S for b in batches) * prof_steps
     kid = 0 if prof_ms[0] >= prof_ms[1] else 1
     kname = "persistent fused step" if fused else ("fine column kernel", "fine row kernel")[kid]
     kbytes = (col_b, row_b)[kid]
@@ -1160,12 +1198,11 @@ def run_parareal(args):
 # kernels, from one ncu capture of the 768-point plan (6, 7) at 1024^2 x 16 slices
 # (one fine step: the 4 stage launches of each kernel), averaged over the stages and
 # scaled by 16 to a 256-slice launch (the traffic grows with the slices); keyed by the
-# kernel's name as the bench reports it and its variant (column variant for the column
-# kernel, row variant for the row kernel).  A variant without a capture of its current
-# code reports null.
+# kernel's name as the bench reports it and the plan (its two variants step on 768 points
+# only as a pair).  A plan without a capture of its current code reports null.
 FINE_TRAFFIC = {
-    ("fine row kernel", 7): 16 * (708.23 + 1067.68 + 888.26 + 867.54) / 4 * 1e6,
-    ("fine column kernel", 6): 16 * (362.56 + 362.71 + 362.48 + 362.83) / 4 * 1e6,
+    ("fine row kernel", (6, 7)): 16 * (708.23 + 1067.68 + 888.26 + 867.54) / 4 * 1e6,
+    ("fine column kernel", (6, 7)): 16 * (362.56 + 362.71 + 362.48 + 362.83) / 4 * 1e6,
 }
 
 
@@ -1211,7 +1248,7 @@ def run_fine_step(args):
     torch.cuda.synchronize()
     prof_ms, prof_n = kd.kd_profile_read(ctx)
     kd.kd_profile(ctx, 0)
-    cb, rb = col_row_bytes(n, B)
+    cb, rb = col_row_bytes(n, B, plan)
     hbm_peak, peak_kind = peaks()
     kid = 0 if prof_ms[0] >= prof_ms[1] else 1
     kname = ("fine column kernel", "fine row kernel")[kid]
@@ -1220,7 +1257,7 @@ def run_fine_step(args):
     achieved = kbytes / (avg_us / 1e6) / 1e9
     stage_ms = (prof_ms[0] + prof_ms[1]) / prof_calls
     stage_bytes = 4 * (cb + rb) * W["steps_per_call"]
-    traffic = FINE_TRAFFIC.get((kname, plan[kid]))
+    traffic = FINE_TRAFFIC.get((kname, tuple(plan)))
 
     # ---- a longer call: the same kernels over 8 steps (the conversions amortised)
     x2 = x_dev.clone()

@@ -69,6 +69,8 @@ static void launch_k(void (*k)(KArgs...), unsigned grid, unsigned block, size_t 
 template <typename T, int R>
 struct FineMrSet {
   static constexpr int N = 32 * R;
+  // the sides of their own (R = 3, 5, 6) step RK443 in kd_fused.cu
+  static constexpr bool RK443 = (R & (R - 1)) == 0;
   static constexpr bool narrow(int, int, int) { return false; }
   static constexpr unsigned BLOCK = 32 * kMrWarps;
   static int ncol() { return 1; }
@@ -86,12 +88,12 @@ struct FineMrSet {
     if (a.scheme == SCHEME_RK111) return row_k<SCHEME_RK111, 0>(a, store, st, pdl);
     if (a.scheme == SCHEME_RK222)
       return mode == 0 ? row_k<SCHEME_RK222, 0>(a, store, st, pdl) : row_k<SCHEME_RK222, 1>(a, store, st, pdl);
-    switch (mode) {
-      case 0: return row_k<SCHEME_RK443, 0>(a, store, st, pdl);
-      case 1: return row_k<SCHEME_RK443, 1>(a, store, st, pdl);
-      case 2: return row_k<SCHEME_RK443, 2>(a, store, st, pdl);
-      default: return row_k<SCHEME_RK443, 3>(a, store, st, pdl);
-    }
+    if constexpr (RK443) switch (mode) {
+        case 0: return row_k<SCHEME_RK443, 0>(a, store, st, pdl);
+        case 1: return row_k<SCHEME_RK443, 1>(a, store, st, pdl);
+        case 2: return row_k<SCHEME_RK443, 2>(a, store, st, pdl);
+        default: return row_k<SCHEME_RK443, 3>(a, store, st, pdl);
+      }
   }
 };
 
@@ -277,6 +279,7 @@ struct Fine2Set {
   using Sh = Shapes2<T, N>;
   using ShC = ShapesC<N>;
   static constexpr bool WIDE = sizeof(T) == 4;
+  static constexpr bool RK443 = WIDE || N == 256;   // the other complex128 sides step it in kd_fused.cu
   static constexpr bool R8 = WIDE && (N == 128 || N == 256);
   // one column variant of every complex64 side is the persistent fused step (kd_fused.cu, taken
   // before these kernels are asked; the row variant does not apply): fused_col(N); the calls
@@ -307,16 +310,16 @@ struct Fine2Set {
   static cudaError_t prepare() {
     cudaError_t e;
     if ((e = prepare_col2<T, N, Sh::xt(0)>()) != cudaSuccess) return e;
-    if ((e = prepare_row2<T, N, Sh::rt(0), true>()) != cudaSuccess) return e;
+    if constexpr (RK443) {
+      if ((e = prepare_row2<T, N, Sh::rt(0), true>()) != cudaSuccess) return e;
+    }
     if ((e = prepare_row2<T, N, Sh::rt(0), true, SCHEME_RK222>()) != cudaSuccess) return e;
     if ((e = prepare_row2<T, N, Sh::rt(0), true, SCHEME_RK111>()) != cudaSuccess) return e;
-    if (WIDE) {
+    if constexpr (WIDE) {
       if ((e = prepare_col2<T, N, Sh::xt(1)>()) != cudaSuccess) return e;
       if ((e = prepare_row2<T, N, Sh::rt(1), true>()) != cudaSuccess) return e;
       if ((e = prepare_row2<T, N, Sh::rt(0), false>()) != cudaSuccess) return e;
       if ((e = prepare_row2<T, N, Sh::rt(1), false>()) != cudaSuccess) return e;
-    }
-    if constexpr (WIDE) {
       if ((e = cudaFuncSetAttribute(col2c_kernel<T, N, ShC::XT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)Col2C<T, N, ShC::XT>::smem)) != cudaSuccess)
         return e;
@@ -376,12 +379,12 @@ struct Fine2Set {
       if (v == 6) return launch_row3<T, N, Shapes8<N>::RT, true, 8>(a, mode, store, st, pdl);
       if (v == 7) return launch_row3<T, N, Shapes8<N>::RT, false, 8>(a, mode, store, st, pdl);
     }
-    switch (v) {
-      case 1: launch_row2<T, N, Sh::rt(1), true>(a, mode, store, st, pdl); break;
-      case 2: launch_row2<T, N, Sh::rt(0), false>(a, mode, store, st, pdl); break;
-      case 3: launch_row2<T, N, Sh::rt(1), false>(a, mode, store, st, pdl); break;
-      default: launch_row2<T, N, Sh::rt(0), true>(a, mode, store, st, pdl); break;
-    }
+    if constexpr (WIDE) switch (v) {
+        case 1: return launch_row2<T, N, Sh::rt(1), true>(a, mode, store, st, pdl);
+        case 2: return launch_row2<T, N, Sh::rt(0), false>(a, mode, store, st, pdl);
+        case 3: return launch_row2<T, N, Sh::rt(1), false>(a, mode, store, st, pdl);
+      }
+    if constexpr (RK443) launch_row2<T, N, Sh::rt(0), true>(a, mode, store, st, pdl);
   }
 };
 
@@ -633,6 +636,7 @@ static int run_steps(const FineArgs& a0, const StepCfg& cfg) {
 
 template <typename T, int N>
 int fine2_run(const FineArgs& a, const StepCfg& cfg) {
+  if (!Fine2Set<T, N>::RK443 && a.scheme == SCHEME_RK443) return -1;   // fine_run took kd_fused.cu
   return run_steps<Fine2Set<T, N>>(a, cfg);
 }
 

@@ -22,7 +22,7 @@ namespace kd {
 template <int N>
 struct NarrowGrid {
   static_assert(N == 768 || N == 384, "3/4 of 1024 and 512");
-  using W = WT<float, 24, N / 24>;
+  using W = WT<N / 24>;
   static constexpr int FULL = N / 3 * 4;               // the problem's grid side
   static constexpr int K = FULL / 3, P = 2 * K + 1;
   static_assert(N >= 2 * K + 2, "no aliasing onto the kept set");
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(ColN<N, GR>::BLOCK, 1) coln_kernel(FineArgs a,
       const cx<float>* buf = In + (k & 1) * P * XG;
       cx<float> s[W::SV];
 #pragma unroll
-      for (int r = 0; r < W::RN; ++r) {
+      for (int r = 0; r < W::C; ++r) {
         const cx<float>* col = buf + CN::in_at(sl + K, wl * C + r);
 #pragma unroll
         for (int q = 0; q < S; ++q) s[r * S + q] = NG::keeps(q, sl) ? col[NG::kofs(q) * XG] : mk(0.f, 0.f);
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(ColN<N, GR>::BLOCK, 1) coln_kernel(FineArgs a,
       W::template p2s<-1>(v, s, lane, B, s_tw);
       named_bar(1 + grp, GT);   // the group's transposes are done: their buffers take the output
 #pragma unroll
-      for (int r = 0; r < W::RN; ++r) {
+      for (int r = 0; r < W::C; ++r) {
         cx<float>* col = Out + (sl + K) * OP + wl * C + r;
 #pragma unroll
         for (int q = 0; q < S; ++q)
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(RowN<N, MODE>::BLOCK, RowN<N, MODE>::MINB) row
   const int c1 = c == 2 ? 0 : c + 1, c2 = c == 0 ? 2 : c - 1, sl = W::slane(lane);
   cx<float>* Sm = (cx<float>*)smem_raw;
   cx<float>* B = Sm + c * RN::WSM;
-  cx<float>* Q = B + W::BUF;                               // [NPRE][SLOTS][32]
+  cx<float>* Q = B + W::BUF;                               // [NST][SLOTS][32]: the staged array, then the stage value
   cx<float>* s_tw = Sm + 3 * RN::WSM;
   W::table(s_tw);
   __syncthreads();
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(RowN<N, MODE>::BLOCK, RowN<N, MODE>::MINB) row
       for (int p = 0; p < V; ++p) v[p] = Wr[S * p];
       W::template p2s<-1>(v, s, lane, B, s_tw);            // x -> kx
 #pragma unroll
-      for (int r = 0; r < W::RN; ++r)
+      for (int r = 0; r < W::C; ++r)
 #pragma unroll
         for (int k = 0; k < S; ++k)
           if (NG::keeps(k, sl)) B[r * P + sl + K + NG::kofs(k)] = s[r * S + k];
@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(RowN<N, MODE>::BLOCK, RowN<N, MODE>::MINB) row
     __syncwarp();
     const cx<float>* X = MODE == 4 ? B : Q;                // the new stage value in wavenumber order
 #pragma unroll
-    for (int r = 0; r < W::RN; ++r)
+    for (int r = 0; r < W::C; ++r)
 #pragma unroll
       for (int k = 0; k < S; ++k)
         s[r * S + k] = NG::keeps(k, sl) ? X[r * P + sl + K + NG::kofs(k)] : mk(0.f, 0.f);

@@ -1,6 +1,6 @@
-// Warp transforms of N = V S points (V = 24 or 12 values a lane in physical space), the
-// sides m = 24 .. 768 = 3/4 of a power of two on which the 2/3-rule step of a power-of-two
-// grid is evaluated.
+// Complex64 warp transforms of N = V S points (V = 24 values a lane in physical space), the sides
+// m = 384 and 768 = 3/4 of 512 and 1024 on which the 2/3-rule step of these grids is evaluated; and
+// the twiddles and small DFTs that kd_fused.cuh shares.
 //
 // Why three quarters.  The kept set is |k| <= K = n / 3 and both flows hold only the
 // wavenumbers +-1, so u x b has |k| <= K + 1 and m >= 2K + 2 points resolve its kept modes
@@ -11,8 +11,8 @@
 //
 // A warp owns C = 32 / S transforms of one kind (columns or rows) at a time:
 //   physical layout: lane l = c S + m1 holds X_c[m1 + S m2], m2 < V          (all 32 lanes)
-//   spectral layout: lanes l < 24 (the rest repeat lane 23); round r < RN: transform c = r CR + l / V, a = l mod V,
-//                    register r S + k holds x_c[a + V k], k < S
+//   spectral layout: lane a < 24 (the rest repeat lane 23), transform r < C: register r S + k holds
+//                    x_r[a + V k], k < S
 // spectral -> physical (n = a + V k, m = m1 + S m2): an S-point DFT over k in the lane, the
 // twiddle w_N^(a m1), a transpose through the warp's shared buffer, a V-point DFT over a.
 // physical -> spectral is the transposed sequence.  One transpose a transform; the S-point
@@ -101,153 +101,117 @@ __device__ __forceinline__ void wt_dft3(cx<T>& a, cx<T>& b, cx<T>& c) {
   c = mk(m.x + h * d.y, m.y - h * d.x);
 }
 
-// V-point DFT of 24 = 3 x 8 or 12 = 3 x 4 points (coprime factors: no twiddles between
-// them).  In: v[n] natural order; out: X[k] at v[wt_pos<V>(k)].
-// Input n = (Q n1 + 3 n2) mod V, output k = k1 mod 3 = k2 mod Q.
-template <int V>
-__host__ __device__ constexpr int wt_pos(int k) {
-  constexpr int Q = V / 3;
-  return (Q * (k % 3) + 3 * bitrev<Q>(k % Q)) % V;
-}
-template <typename T, int V, int DIR>
-__device__ __forceinline__ void wt_dftv(cx<T> (&v)[V]) {
-  static_assert(V == 24 || V == 12, "3 x 8 or 3 x 4");
-  constexpr int Q = V / 3;
+// DFT of 24 = 3 x 8 points (coprime factors: no twiddles between them).  In: v[n] natural
+// order; out: X[k] at v[wt_pos(k)].  Input n = (8 n1 + 3 n2) mod 24, output k = k1 mod 3 = k2 mod 8.
+__host__ __device__ constexpr int wt_pos(int k) { return (8 * (k % 3) + 3 * bitrev<8>(k % 8)) % 24; }
+template <int DIR>
+__device__ __forceinline__ void wt_dft24(cx<float> (&v)[24]) {
 #pragma unroll
-  for (int n2 = 0; n2 < Q; ++n2)
-    wt_dft3<T, DIR>(v[(3 * n2) % V], v[(Q + 3 * n2) % V], v[(2 * Q + 3 * n2) % V]);
+  for (int n2 = 0; n2 < 8; ++n2)
+    wt_dft3<float, DIR>(v[(3 * n2) % 24], v[(8 + 3 * n2) % 24], v[(16 + 3 * n2) % 24]);
 #pragma unroll
   for (int k1 = 0; k1 < 3; ++k1) {
-    cx<T> u[Q];
+    cx<float> u[8];
 #pragma unroll
-    for (int n2 = 0; n2 < Q; ++n2) u[n2] = v[(Q * k1 + 3 * n2) % V];
-    dft_dif<T, Q, DIR>(u);                             // residue k2 at u[bitrev(k2)]
+    for (int n2 = 0; n2 < 8; ++n2) u[n2] = v[(8 * k1 + 3 * n2) % 24];
+    dft_dif<float, 8, DIR>(u);                         // residue k2 at u[bitrev(k2)]
 #pragma unroll
-    for (int n2 = 0; n2 < Q; ++n2) v[(Q * k1 + 3 * n2) % V] = u[n2];
+    for (int n2 = 0; n2 < 8; ++n2) v[(8 * k1 + 3 * n2) % 24] = u[n2];
   }
 }
 
-// In-lane S-point DFT, natural order in; X[k] at v[bitrev<S>(k)].
-template <typename T, int S, int DIR>
-__device__ __forceinline__ void wt_dfts(cx<T>* v) {
-  if constexpr (S > 1) dft_dif<T, S, DIR>(v);
-}
-
-template <typename T, int V_, int S_>
+template <int S_>
 struct WT {
-  static_assert((V_ == 24 || V_ == 12) && S_ >= 1 && S_ <= 32, "values a lane, lanes a transform");
-  static constexpr int V = V_, S = S_, N = V * S;
+  static_assert(S_ == 32 || S_ == 16, "lanes a transform");
+  static constexpr int V = 24, S = S_, N = V * S;
   static constexpr int C = 32 / S;                     // transforms of a warp
-  static constexpr int CR = 24 / V;                    // transforms of a spectral round
-  static constexpr int RN = C / CR;                    // spectral rounds
-  static_assert(C % CR == 0, "whole rounds");
-  static constexpr int SV = RN * S;                    // spectral values a lane
-  // transpose buffer: [c][m1][a], rows of PITCH complex.  PITCH makes the 16-byte row
-  // accesses of a quarter warp conflict-free; CPAD puts the two transforms of a spectral
-  // round on different banks (V = 12).
-  static constexpr int PITCH = sizeof(T) == 4 ? V + 2 : V + 1;
-  static constexpr int CPAD = V == 12 ? 12 : 0;
-  static constexpr int CST = S * PITCH + CPAD;         // complex per transform
+  static constexpr int SV = C * S;                     // spectral values a lane
+  // transpose buffer: [c][m1][a], rows of PITCH complex: the 16-byte row accesses of a quarter
+  // warp are conflict-free
+  static constexpr int PITCH = V + 2;
+  static constexpr int CST = S * PITCH;                // complex per transform
   static constexpr int BUF = C * CST;
   // twiddles of a lane: w_N^(a m1) from the table s_tw[m1 * V + a] (m1 < S)
   static constexpr int TAB = S * V;
 
-  static __device__ __forceinline__ void table(cx<T>* s_tw) {
-    for (int i = threadIdx.x; i < TAB; i += blockDim.x) s_tw[i] = wt_tw<N, T>(((i / V) * (i % V)) % N);
+  static __device__ __forceinline__ void table(cx<float>* s_tw) {
+    for (int i = threadIdx.x; i < TAB; i += blockDim.x) s_tw[i] = wt_tw<N, float>(((i / V) * (i % V)) % N);
   }
   // The spectral lane of lane l: lanes 24..31 read and compute what lane 23 does (their values are
   // not stored), which costs no more than idling them and keeps the code free of divergence.
   static __device__ __forceinline__ int slane(int l) { return l < 24 ? l : 23; }
-  // transform and element of spectral register (round r, k) in spectral lane l
-  static __device__ __forceinline__ int spec_c(int l, int r) { return CR == 1 ? r : 2 * r + (l >= V ? 1 : 0); }
-  static __device__ __forceinline__ int spec_a(int l) { return CR == 1 ? l : (l >= V ? l - V : l); }
   static __device__ __forceinline__ int phys_c(int l) { return l / S; }
   static __device__ __forceinline__ int phys_m1(int l) { return l % S; }
 
   template <int DIR>
-  static __device__ __forceinline__ cx<T> tw_mul(cx<T> v, cx<T> w) {
+  static __device__ __forceinline__ cx<float> tw_mul(cx<float> v, cx<float> w) {
     return DIR < 0 ? mk(v.x * w.x - v.y * w.y, v.x * w.y + v.y * w.x) : mk(v.x * w.x + v.y * w.y, v.y * w.x - v.x * w.y);
   }
 
   // Spectral registers s -> physical registers v.  B: the warp's buffer (BUF complex), free on
   // entry; free again on return for accesses after a __syncwarp.
   template <int DIR>
-  static __device__ __forceinline__ void s2p(cx<T> (&s)[SV], cx<T> (&v)[V], int l, cx<T>* B, const cx<T>* s_tw) {
-    const int sl = slane(l), a = spec_a(sl);
+  static __device__ __forceinline__ void s2p(cx<float> (&s)[SV], cx<float> (&v)[V], int l, cx<float>* B,
+                                             const cx<float>* s_tw) {
+    const int a = slane(l);
 #pragma unroll
-    for (int r = 0; r < RN; ++r) {
-      wt_dfts<T, S, DIR>(&s[r * S]);
-      cx<T>* row = B + spec_c(sl, r) * CST + a;
+    for (int r = 0; r < C; ++r) {
+      dft_dif<float, S, DIR>(&s[r * S]);               // X[m1] at bitrev(m1)
+      cx<float>* row = B + r * CST + a;
 #pragma unroll
       for (int m1 = 0; m1 < S; ++m1) {
-        cx<T> y = s[r * S + bitrev<S>(m1)];
+        cx<float> y = s[r * S + bitrev<S>(m1)];
         if (m1 != 0) y = tw_mul<DIR>(y, s_tw[m1 * V + a]);
         if (l < 24) row[m1 * PITCH] = y;
       }
     }
     __syncwarp();
-    const cx<T>* row = B + phys_c(l) * CST + phys_m1(l) * PITCH;
-    load_row(row, v);
-    __syncwarp();
-    wt_dftv<T, V, DIR>(v);
-    cx<T> t[V];
+    const cx<float>* row = B + phys_c(l) * CST + phys_m1(l) * PITCH;
 #pragma unroll
-    for (int k = 0; k < V; ++k) t[k] = v[wt_pos<V>(k)];
+    for (int i = 0; i < V; i += 2) {
+      const float4 q = *(const float4*)&row[i];
+      v[i] = mk(q.x, q.y);
+      v[i + 1] = mk(q.z, q.w);
+    }
+    __syncwarp();
+    wt_dft24<DIR>(v);
+    cx<float> t[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) t[k] = v[wt_pos(k)];
 #pragma unroll
     for (int k = 0; k < V; ++k) v[k] = t[k];
   }
 
   // Physical registers v (destroyed) -> spectral registers s.
   template <int DIR>
-  static __device__ __forceinline__ void p2s(cx<T> (&v)[V], cx<T> (&s)[SV], int l, cx<T>* B, const cx<T>* s_tw) {
-    wt_dftv<T, V, DIR>(v);                             // residue a at v[wt_pos(a)]
-    store_row(B + phys_c(l) * CST + phys_m1(l) * PITCH, v);
-    __syncwarp();
-    const int sl = slane(l), a = spec_a(sl);
+  static __device__ __forceinline__ void p2s(cx<float> (&v)[V], cx<float> (&s)[SV], int l, cx<float>* B,
+                                             const cx<float>* s_tw) {
+    wt_dft24<DIR>(v);                                  // residue a at v[wt_pos(a)]
+    cx<float>* to = B + phys_c(l) * CST + phys_m1(l) * PITCH;
 #pragma unroll
-    for (int r = 0; r < RN; ++r) {
-      const cx<T>* row = B + spec_c(sl, r) * CST + a;
+    for (int i = 0; i < V; i += 2) {
+      const cx<float> y0 = v[wt_pos(i)], y1 = v[wt_pos(i + 1)];
+      *(float4*)&to[i] = make_float4(y0.x, y0.y, y1.x, y1.y);
+    }
+    __syncwarp();
+    const int a = slane(l);
+#pragma unroll
+    for (int r = 0; r < C; ++r) {
+      const cx<float>* row = B + r * CST + a;
 #pragma unroll
       for (int m1 = 0; m1 < S; ++m1) {
-        cx<T> y = row[m1 * PITCH];
+        cx<float> y = row[m1 * PITCH];
         if (m1 != 0) y = tw_mul<DIR>(y, s_tw[m1 * V + a]);
         s[r * S + m1] = y;
       }
-      wt_dfts<T, S, DIR>(&s[r * S]);
-      cx<T> t[S];
+      dft_dif<float, S, DIR>(&s[r * S]);
+      cx<float> t[S];
 #pragma unroll
       for (int k = 0; k < S; ++k) t[k] = s[r * S + bitrev<S>(k)];
 #pragma unroll
       for (int k = 0; k < S; ++k) s[r * S + k] = t[k];
     }
     __syncwarp();
-  }
-
- private:
-  static __device__ __forceinline__ void load_row(const cx<T>* row, cx<T> (&v)[V]) {
-    if constexpr (sizeof(T) == 4) {
-#pragma unroll
-      for (int a = 0; a < V; a += 2) {
-        const float4 q = *(const float4*)&row[a];
-        v[a] = mk((T)q.x, (T)q.y);
-        v[a + 1] = mk((T)q.z, (T)q.w);
-      }
-    } else {
-#pragma unroll
-      for (int a = 0; a < V; ++a) v[a] = row[a];
-    }
-  }
-  static __device__ __forceinline__ void store_row(cx<T>* row, const cx<T> (&v)[V]) {
-    if constexpr (sizeof(T) == 4) {
-#pragma unroll
-      for (int a = 0; a < V; a += 2) {
-        const cx<T> y0 = v[wt_pos<V>(a)], y1 = v[wt_pos<V>(a + 1)];
-        *(float4*)&row[a] = make_float4((float)y0.x, (float)y0.y, (float)y1.x, (float)y1.y);
-      }
-    } else {
-#pragma unroll
-      for (int a = 0; a < V; ++a) row[a] = v[wt_pos<V>(a)];
-    }
   }
 };
 

@@ -556,15 +556,13 @@ __global__ void __launch_bounds__(TB) k_grad_norm(const float* W, const float* W
   constexpr int U = 4;                                       // tiles of TB columns of a row in flight
   float s0 = 0.f, s1 = 0.f, s2 = 0.f;                        // the sum so far: s0 + s1 + s2
   double far = 0.0;
-  const int chunks = (nc + TB - 1) / TB;
-  const long tiles = (long)rows * chunks;
-  for (long t0 = blockIdx.x; t0 < tiles; t0 += (long)U * gridDim.x) {
+  const int chunks = (nc + TB - 1) / TB, tiles = rows * chunks;   // 1.2 million at 64 modes
+  for (int t0 = blockIdx.x; t0 < tiles; t0 += U * (int)gridDim.x) {
     long at[U];
     float w[U], w0[U], g[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const long t = t0 + (long)u * gridDim.x;
-      const int row = (int)(t / chunks), j = (int)(t - (long)row * chunks) * TB + threadIdx.x;
+      const int t = t0 + u * (int)gridDim.x, row = t / chunks, j = (t - row * chunks) * TB + (int)threadIdx.x;
       const bool in = t < tiles && j < nc;
       at[u] = in ? (long)row * nc + j : -1;
       w[u] = in ? W[at[u]] : 0.f;

@@ -161,6 +161,15 @@ bool grid_of(kd_ctx* ctx, int grid, int* n, int* prec) {
   return true;
 }
 
+// Whether the pair runs the kernels of another candidate: the persistent step, which has no row kernel,
+// with another row variant, or, at a scheme it does not have, another column variant's kernel; and the
+// second name of the 512-point column kernel, which stands for it where the first is half of a 3n/4 pair.
+bool same_kernels(int n, int prec, int scheme, int col, int row) {
+  if (prec != KD_C64) return false;
+  if (n <= 256 && col == fused_col(n)) return row > 0 || !fused_covers(n / 3, scheme);
+  return n == 512 && col == 6 && (row != 9 || scheme != KD_RK443);
+}
+
 // The plan of a grid from now on, for calls of every batch.
 void choose(kd_ctx* ctx, int grid, int col, int row) {
   ctx->plan[grid].col = col;
@@ -283,8 +292,7 @@ kd_status kd_autotune(kd_ctx* ctx, int grid, int batch, int nsteps, const char* 
   FinePlan best_plan = saved;
   for (int c = 0; c < nc && s == KD_OK; ++c)
     for (int r = 0; r < nr && s == KD_OK; ++r) {
-      // the persistent fused step has no row kernel: one candidate
-      if (r > 0 && prec == KD_C64 && c == fused_col(n) && fused_covers(n / 3, a.scheme)) continue;
+      if (same_kernels(n, prec, a.scheme, c, r)) continue;
       ctx->plan[grid].col = c;
       ctx->plan[grid].row = r;
       if (fill_hash(prec, w.X, (long)batch * compact_len(n), 12345u, ctx->st) < 0 ||

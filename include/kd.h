@@ -78,9 +78,12 @@ typedef struct {
                           n = 16, 32, ..., 1024 or any other even n <= 286.  The flow has only
                           the wavenumbers +-1, so any m >= 2 (n/3) + 2 points resolve u x b on
                           the kept set without aliasing, exactly as n points do, and RK443
-                          steps transform on such an m: 24, 32, 48, 96, 128 or 192 for n <= 286,
+                          steps transform on such an m: 16, 24, 32, 48, 96, 128 or 192 for n <= 286,
                           3n/4 for n = 512 and 1024 in complex64 (n = 240, the 3/2-padded grid
-                          of 160 kept modes, runs on 192); complex128 n = 256, 512 and 1024,
+                          of 160 kept modes, runs on 192).  Round-off is spread over m^2
+                          points: a complex64 step of a power-of-two side on 3n/4 points errs by
+                          1.15 to 1.27 times (at most 4/3) the n-point one, which kd_set_plan
+                          with (0, 0) selects.  complex128 n = 256, 512 and 1024,
                           launch plans other than the default, RK222 and RK111 on n
                           itself or, where n is neither a power of two nor 96, 160, 192, on the
                           smallest of these three that suffices.  KD_FINE_CONV: even
@@ -265,9 +268,10 @@ kd_status kd_set_coarse_sync(kd_ctx* ctx, int mode);
  * the sweep has passed its last slice, and the next sweep waits for each chunk before its
  * first slice.  The parallel step is computed before the defect of iteration k is known
  * and discarded if the run stops there.  The results are those of the unpipelined order
- * bit for bit.  It pays when a chunk's fine work is few launches (KD_FINE_CONV); with the
- * FFT operator every chunk repeats all the step launches on a smaller batch.  KD_EINVAL
- * for chunks outside [0, 16]. */
+ * bit for bit.  The chunks follow one another, each over all its steps on a part of the
+ * slices, beside a sweep that uses few SMs: at 128^2 with 64 slices two chunks gain (FFT
+ * operator 56.4 -> 49.6 ms a solve) and more lose (4: 62.0, 8: 118.1; KD_FINE_CONV 40.5 ms
+ * with 0, 41.2, 44.7, 45.8 with 2, 4, 8).  KD_EINVAL for chunks outside [0, 16]. */
 kd_status kd_set_overlap(kd_ctx* ctx, int chunks);
 
 /* Serial fine solution at the slice boundaries, U_{n+1} = F(U_n) with each slice
@@ -454,7 +458,8 @@ kd_status kd_gemm_bf16_tn(const void* A, const void* Bt, float* C, int M, int N,
                           void* cuda_stream);
 
 /* CUDA graphs for the Parareal fine sweeps of the FFT operator (default on; not used
- * with kd_set_overlap's pipelined iterations): the ~8 S launches of one sweep shape
+ * with kd_set_overlap's pipelined iterations): the launches of one sweep shape (four, or
+ * ~8 S where the step takes two kernels a stage)
  * (first slice, slices, steps, step, form, launch plan) are captured once into a graph
  * and replayed on a stream of the context, fenced by events against the context stream;
  * any device allocation of the context invalidates the captured graphs.  Off: direct
@@ -477,15 +482,15 @@ kd_status kd_selftest_wait(int arrive, double max_ms, void* cuda_stream);
  * tables, fine and coarse workspaces, Parareal arrays, staging; not CUDA's own objects
  * such as streams, events and graph executables, nor the static array of
  * kd_fine_batched_static).  Training buffers that the context keeps for its next training
- * call (at most 1 GiB, the newest) count as held and are released
- * before a request is refused; on a GPU that is out of memory those of every context are
- * released before a request of any fails.  Other allocators of the process (PyTorch) cannot
- * ask for them: kd_destroy gives a context's back.  max_bytes = 0 removes the limit (the
- * default); a limit below what the context already holds keeps the buffers in use and
- * refuses new ones.  A call that needs a
- * buffer beyond the limit returns KD_ENOMEM, as a failed cudaMalloc does, with
- * kd_last_error naming the buffer, its size, the bytes held and the limit; the context
- * stays usable, and the same call succeeds once the limit allows it.  Contexts that
+ * call (at most 1 GiB, the newest) count as held and are released before a request is
+ * refused; on a GPU that is out of memory those of every context are released before a
+ * request of any fails.  Other allocators of the process (PyTorch) cannot ask for them:
+ * kd_destroy gives a context's back.  max_bytes = 0 removes the limit (the default); a
+ * limit below what the context already holds keeps the buffers in use and refuses new
+ * ones.  A call that needs a buffer beyond the limit returns KD_ENOMEM, as a failed
+ * cudaMalloc does, with kd_last_error naming the buffer, its size, the bytes held and the
+ * limit; the context stays usable, and the same call succeeds once the limit allows it.
+ * Contexts that
  * kd_sweep_create makes for itself are not affected.  kd_get_alloc_bytes returns the bytes
  * held and the limit (either pointer may be NULL).  Both are host-only: no CUDA call. */
 kd_status kd_set_alloc_limit(kd_ctx* ctx, size_t max_bytes);

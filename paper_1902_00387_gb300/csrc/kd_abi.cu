@@ -644,8 +644,8 @@ kd_status run_graph(kd_ctx* ctx, const std::string& key, const std::function<kd_
   return KD_OK;
 }
 
-// The FFT operator's fine sweep is ~8 S + 3 launches; with graphs on, the launches of
-// one sweep shape are captured once into a CUDA graph (programmatic dependent launches
+// The FFT operator's fine sweep is four launches, or ~8 S + 3 where the step takes two kernels a
+// stage; with graphs on, the launches of one sweep shape are captured once into a CUDA graph (programmatic dependent launches
 // included) and replayed; the values are those of the direct launches.
 kd_status fine_sweep(kd_ctx* ctx, int first, int N, int S, double dt, int iter, long whole) {
   const FinePlan plan = call_plan(ctx, whole);

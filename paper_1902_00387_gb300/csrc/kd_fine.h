@@ -50,6 +50,7 @@ bool fine_variants(int n, int prec, int* ncol, int* nrow);
 // fine_few(n) fields (and for the coarse grid, whose serial sweep steps one at a time), which
 // leave most of the GPU idle in the default's larger blocks
 FinePlan fine_default_plan(int n, int prec, bool few = false);
+// where the two cross:
 //   n = 256, (6, 0) | (0, 9), us a step of 1, 3, 4, 6 fields: 58.9 59.3 58.7 59.0 | 47.7 54.4 59.1 65.3
 //   n = 512, (5, 9) | (6, 9), of 1, 2, 3, 4 fields: 86.0 92.9 98.0 118.1 | 71.7 80.2 121.4 133.2
 constexpr int fine_few(int n, int prec) { return prec != 0 ? 0 : (n == 256 ? 4 : (n == 512 ? 2 : 0)); }
@@ -63,7 +64,7 @@ bool fine_full_io(int n, int prec, const FinePlan& plan, int scheme);
 // a.phases (which must hold phase_table_bytes(prec, a.batch, nsteps)).  Returns the
 // number of kernels launched (negative on an unsupported grid size).
 int fine_run(int prec, const FineArgs& a, const StepCfg& cfg);
-// the same with the default plan and every field taking every step
+// the same with plan {0, 0} and every field taking every step
 int fine_launch_steps(int prec, const FineArgs& a, int nsteps, bool prologue, bool store_last,
                       cudaStream_t st, const LaunchProbe* probe = nullptr);
 

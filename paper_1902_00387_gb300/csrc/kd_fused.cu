@@ -23,7 +23,7 @@ struct LaneKernel {
   using F = FusedStep<T, L, R>;
   static constexpr auto kernel = fused_kernel<T, L, R>;
   // Fields for which the passes run as launches of their own (0: never).  An SM has few FP64 units
-  // and a field has 16 SMs at most in a cluster, so that up to nine fields take what one takes.  192^2
+  // and a field has 16 SMs at most in a cluster, so that up to seven fields take what one takes.  192^2
   // complex128, us a step of 1, 4, 8, 12, 24 fields, clusters | launches: 1070 1072 1323 2071 4131 |
   // 640 776 1007 1334 2616.  More fields gain less (40: 4934 | 4140), for room in W that grows with them.
   // In complex64 the launches' latencies take what the units would give (54 55 75 88 141 | 49 56 81

@@ -309,10 +309,12 @@ __device__ __forceinline__ cx<T> fused_update(cx<T>* o0, cx<T>* o1, cx<T>* o2, b
 // Xlo when s0 > 0) back to X (Xlo).
 //
 // A few fields of the largest complex128 sets leave most of the GPU idle in clusters, 16 SMs each at
-// most.  For them (LaneKernel::SPREAD in kd_fused.cu) the same passes run as launches over the whole GPU, a warp a block, with the mixed field in global memory (a.W, L2):
-// FUSED_COLS: column pass of stage nsteps of step s0, field blockIdx.y; FUSED_ROWS: row pass (4:
-// before the first stage), CS: whether another stage follows.  The arithmetic is this one source's,
-// so the values are the same bits.
+// most, and FP64 arithmetic bounds them.  For them (LaneKernel::SPREAD in kd_fused.cu, with the
+// times of both) the same passes run as launches over the whole GPU, a warp a block, so that every
+// quarter of an SM has one task, with the mixed field in global memory (a.W, L2).  FUSED_COLS: column
+// pass of stage nsteps of step s0, field blockIdx.y; FUSED_ROWS: row pass of stage nsteps (4: before the
+// first stage), CS: whether another stage follows.  The arithmetic is this one source's, so the
+// values are the same bits.
 enum { FUSED_CLUSTER = 0, FUSED_COLS = 1, FUSED_ROWS = 2 };
 
 template <typename T, int L, int R, int MODE = FUSED_CLUSTER>

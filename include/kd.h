@@ -138,8 +138,9 @@ kd_status kd_fine_batched(kd_ctx* ctx, const void* b_in, void* b_out, const doub
  * chunks, the copy in of a chunk, its propagation and the copy out of the previous chunk
  * overlapping on three streams (two device slots per direction, allocated on first use
  * and kept).  chunk > 0: chunks of that many fields (the last one ragged); chunk = 0: a
- * graded plan, chunks doubling from ceil(batch / 32) fields up to batch / 4, then back
- * down (a short pipeline fill and drain, large batches for the steps in between; 8, 16,
+ * graded plan, chunks doubling from ceil(batch / 32) fields (at least 5 at n = 256 and 3
+ * at n = 512 in complex64, of batches that large, where there is room) up to batch / 4, then
+ * back down (a short pipeline fill and drain, large batches for the steps in between; 8, 16,
  * 32, 48, 48, 48, 32, 16, 8 for 256 fields).  Same values as kd_fine_batched, field by
  * field.  No counterpart in the paper (host I/O of this library).
  *   h_in, h_out : host, [batch][3][n][n] complex in params.prec_fine (page-locked memory

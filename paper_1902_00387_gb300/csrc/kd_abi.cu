@@ -16,6 +16,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <complex>
 #include <mutex>
 #include <string>
@@ -1068,18 +1069,18 @@ static kd_status fine_kept(kd_ctx* ctx, const void* c_in, void* c_out, const dou
 }
 
 // Chunk sizes of a host-buffer call.  chunk > 0: equal chunks (the last one ragged).
-// chunk = 0: sizes that double from base = ceil(batch / 32) up to below cap = batch / 4,
-// then equal chunks of at most cap, then the same ramp down: the first copy in and the
-// last copy out (the pipeline's fill and drain) move base fields, while the steps in
+// chunk = 0: sizes that double from base = ceil(batch / 32), `least` if that is more, up to below
+// cap = batch / 4, then equal chunks of at most cap, then the same ramp down: the first copy in
+// and the last copy out (the pipeline's fill and drain) move base fields, while the steps in
 // between run on batches large enough to fill the GPU; every chunk's copies fit under
 // its neighbour's steps.
-static std::vector<int> chunk_plan(int batch, int chunk) {
+static std::vector<int> chunk_plan(int batch, int chunk, int least = 1) {
   std::vector<int> out;
   if (chunk > 0) {
     for (int f = 0; f < batch; f += chunk) out.push_back(batch - f < chunk ? batch - f : chunk);
     return out;
   }
-  const int base = (batch + 31) / 32, cap = batch / 4 > base ? batch / 4 : base;
+  const int base = std::max((batch + 31) / 32, least), cap = batch / 4 > base ? batch / 4 : base;
   std::vector<int> up;
   int ramp = 0;
   for (int c = base; c < cap; c *= 2) {
@@ -1152,7 +1153,7 @@ static kd_status host_chunks_kept(kd_ctx* ctx, const void* h_in, void* h_out, co
 
 // Set-up shared by the host-buffer calls: the four device slots for the largest chunk of
 // `plan` at `slot_field` bytes a field, the start-time array and the copy streams.
-static kd_status host_setup(kd_ctx* ctx, int batch, const std::vector<int>& plan, size_t slot_field) {
+static kd_status host_slots(kd_ctx* ctx, int batch, const std::vector<int>& plan, size_t slot_field) {
   int most = 0;
   for (int c : plan) most = c > most ? c : most;
   const size_t slot = slot_field * most;
@@ -1182,6 +1183,34 @@ static kd_status host_setup(kd_ctx* ctx, int batch, const std::vector<int>& plan
   return KD_OK;
 }
 
+// The chunks and their set-up.  Every chunk steps with the plan of the whole batch, so a batch of more
+// fields than the few-field plan serves moves in chunks of more, too: the plan of many fields takes
+// one to seven fields of 256^2 in one time (16 fields, 3 steps, in chunks of 1, 2, 4, 3, 3, 2, 1
+// 1593 us, in four chunks 957; 6 fields of 512^2 1787 and 918).  Where an allocation limit or the GPU has no room for these chunks, the smaller ones.
+static kd_status host_setup(kd_ctx* ctx, int batch, int chunk, int nsteps, size_t slot_field, std::vector<int>& plan) {
+  const int few = conv_op(ctx) ? 0 : fine_few(ctx->p.n, ctx->p.prec_fine);
+  if (chunk == 0 && few > 0 && batch > few) {
+    plan = chunk_plan(batch, 0, few + 1);
+    kd_status s = host_slots(ctx, batch, plan, slot_field);
+    // the workspace of the largest chunk now, so that nothing is refused once fields have moved
+    const int n = ctx->p.n, most = *std::max_element(plan.begin(), plan.end());
+    if (s == KD_OK) s = ensure_ws(ctx, ctx->ws_f, n, ctx->p.prec_fine, most);
+    if (s == KD_OK) {
+      FineArgs a = fine_args(ctx, ctx->ws_f, ctx->tab_f, n, most, ctx->p.dt_fine, nullptr);
+      s = with_phases(ctx, ctx->ws_f, a, nsteps);
+    }
+    if (s != KD_ENOMEM) return s;
+    for (void*& q : ctx->hio) {
+      dfree(ctx, q);
+      q = nullptr;
+    }
+    ctx->hio_bytes = 0;
+    ctx->ws_f.cap = 0;        // given back by the next request
+  }
+  plan = chunk_plan(batch, chunk);
+  return host_slots(ctx, batch, plan, slot_field);
+}
+
 // Waits for the three streams of a host-buffer call: whatever happened, no copy of the
 // caller's memory is left in flight on return.
 static kd_status host_finish(kd_ctx* ctx, kd_status s, const char* what) {
@@ -1201,8 +1230,8 @@ kd_status kd_fine_batched_host(kd_ctx* ctx, const void* h_in, void* h_out, const
   if (batch == 0) return KD_OK;
   const int n = ctx->p.n;
   const size_t fb = 3 * (size_t)n * n * csize(ctx->p.prec_fine);   // bytes of one field
-  const std::vector<int> plan = chunk_plan(batch, chunk);
-  kd_status s = host_setup(ctx, batch, plan, fb);
+  std::vector<int> plan;
+  kd_status s = host_setup(ctx, batch, chunk, nsteps, fb, plan);
   if (s != KD_OK) return s;
   return host_finish(ctx, host_chunks(ctx, h_in, h_out, t0, nsteps, batch, plan, fb), "kd_fine_batched_host");
 }
@@ -1215,8 +1244,8 @@ kd_status kd_fine_batched_host_kept(kd_ctx* ctx, const void* h_in, void* h_out, 
     return fail(ctx, KD_EINVAL, "kd_fine_batched_host_kept: negative argument");
   if (batch == 0) return KD_OK;
   const size_t fb = compact_len(ctx->p.n) * csize(ctx->p.prec_fine);   // bytes of one field
-  const std::vector<int> plan = chunk_plan(batch, chunk);
-  kd_status s = host_setup(ctx, batch, plan, fb);
+  std::vector<int> plan;
+  kd_status s = host_setup(ctx, batch, chunk, nsteps, fb, plan);
   if (s != KD_OK) return s;
   return host_finish(ctx, host_chunks_kept(ctx, h_in, h_out, t0, nsteps, batch, plan, fb),
                      "kd_fine_batched_host_kept");

@@ -10,7 +10,7 @@
 // (30.2), the column kernel 2.30 a launch; a step of 45 fields of 512^2 1.02 ms (1.38).  With all
 // the stage arrays of a row staged in shared memory (three blocks an SM instead of five at stages
 // 1 and 3) and three accumulators stored by stage 0 the steps took 25.3 and 1.15 ms.  Two column groups
-// a block (8 warps, 255 registers) took 2.32 ms, so a third (12 warps, 168 registers, 160
+// a block (8 warps, 255 registers) took 2.32 ms, so a third (12 warps, 168 registers, 140
 // bytes of spills) gains little; the components in rolled loops (38 instead of 92 KB of
 // code) 2.85 ms, for the register moves and the lost overlap.
 #pragma once

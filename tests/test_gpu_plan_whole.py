@@ -33,7 +33,7 @@ def batched(kd, n, b, t0):
     import torch
     ctx = context(kd, n)
     try:
-        x = torch.tensor(b, dtype=torch.complex64, device="cuda")
+        x = torch.as_tensor(b).to("cuda", torch.complex64)
         y = torch.empty_like(x)
         kd.kd_fine_batched(ctx, x, y, torch.tensor(t0, dtype=torch.float64, device="cuda"), S, len(b))
         torch.cuda.synchronize()
@@ -89,3 +89,27 @@ def test_training_pairs(kd, pairs):
         kd.kd_destroy(ctx)
     ref = batched(kd, n, b, [0.0] * pairs)[:, :, k][:, :, :, k]
     assert np.array_equal(y.cpu().numpy(), ref)
+
+
+# fields and the largest chunk without a lower bound on chunks
+@pytest.mark.parametrize("n,fields,largest", [(256, 5, 1), (256, 16, 4), (512, 3, 1), (512, 9, 2)])
+def test_graded_chunks_of_host_fields(kd, n, fields, largest):
+    """Chunks of a host-buffer call that are larger than a few fields: the device call's bits, also in
+    place and under an allocation limit that has room for the smaller chunks only."""
+    import torch
+    b = torch.tensor(I.initial_batch(n, 0.57, range(fields)), dtype=torch.complex64)
+    t0 = np.arange(fields, dtype=np.float64)
+    ref = batched(kd, n, b, t0)
+    limit = 0
+    for chunk in (largest, 0, 0):
+        ctx = context(kd, n)
+        try:
+            kd.kd_set_alloc_limit(ctx, limit)
+            y = b.clone()
+            kd.kd_fine_batched_host(ctx, y, y, t0, S, fields, chunk)
+            assert np.array_equal(y.numpy(), ref)
+            held = kd.kd_get_alloc_bytes(ctx)[0]
+            assert not limit or held <= limit
+            limit = 0 if chunk == 0 else held
+        finally:
+            kd.kd_destroy(ctx)
